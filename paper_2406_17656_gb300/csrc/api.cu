@@ -682,9 +682,10 @@ __global__ void replicate_cols_kernel(int64_t n, T *a) {
 // n columns, offsets off0[kNumBins + 1]): the maps interleaved column by
 // column, work[K t + k] = work0[t] + k n, off[c] = K off0[c], so that the
 // same column of every map is solved side by side (one block reads map 0's
-// metadata for all of them)
-__global__ void expand_work_kernel(int K, MapChunks ch, int n, const int32_t *work0, const int32_t *off0, int32_t *work,
-                                   int32_t *off) {
+// metadata for all of them); by_map: map by map instead, so that neighbouring
+// lanes of the thread-per-column kernel read neighbouring columns of one map
+__global__ void expand_work_kernel(int K, MapChunks ch, int by_map, int n, const int32_t *work0, const int32_t *off0,
+                                   int32_t *work, int32_t *off) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = blockIdx.y;
     if (t < off0[kNumBins]) {
@@ -696,14 +697,15 @@ __global__ void expand_work_kernel(int K, MapChunks ch, int n, const int32_t *wo
         int q = 0;
         while (q + 1 < ch.count && k >= ch.start[q + 1]) ++q;
         const int k0 = ch.start[q], wq = ch.start[q + 1] - k0;
-        work[(int64_t)K * off0[b] + (int64_t)k0 * c + wq * tl + (k - k0)] = work0[t] + k * n;
+        work[(int64_t)K * off0[b] + (by_map ? (int64_t)k * c + tl : (int64_t)k0 * c + wq * tl + (k - k0))] =
+            work0[t] + k * n;
     }
     if (t <= kNumBins && k == 0) off[t] = K * off0[t];
 }
 
 cudaError_t interleaved_work_list(sam_handle h, Scratch &sc, int K, int n, const uint8_t *bin, int32_t *work,
                                   int32_t *bin_off, const MapChunks *chunks = nullptr,
-                                  const int32_t **off0_out = nullptr) {
+                                  const int32_t **off0_out = nullptr, bool by_map = false) {
     int32_t *work0 = sc.get<int32_t>((size_t)n), *off0 = sc.get<int32_t>(kNumBins + 1);
     if (!work0 || !off0) return cudaErrorMemoryAllocation;
     cudaError_t e = build_work_list(h, n, bin, work0, off0);
@@ -711,7 +713,7 @@ cudaError_t interleaved_work_list(sam_handle h, Scratch &sc, int K, int n, const
     const int64_t cnt = std::max<int64_t>(n, kNumBins + 1);
     dim3 grid((unsigned)((cnt + 255) / 256), (unsigned)K);
     const MapChunks ch = chunks ? *chunks : plan_chunks(K, n, false);
-    expand_work_kernel<<<grid, 256, 0, h->stream>>>(K, ch, n, work0, off0, work, bin_off);
+    expand_work_kernel<<<grid, 256, 0, h->stream>>>(K, ch, by_map ? 1 : 0, n, work0, off0, work, bin_off);
     count_launch(h);
     if (off0_out) *off0_out = off0;
     return cudaGetLastError();
@@ -1333,6 +1335,53 @@ sam_status tape_args(sam_handle h, Scratch &sc, const PatternGroup *g, int64_t N
     return SAM_OK;
 }
 
+// the longest column of K structurally symmetric sources (as long as their
+// rows: mrow, of the validation), -1 when it is not known
+int longest_column(const std::vector<char> &sym, const std::vector<int32_t> &mrow, int K) {
+    int m = 0;
+    for (int k = 0; k < K; ++k) {
+        if (!sym[k] || mrow[k] < 0) return -1;
+        m = std::max(m, (int)mrow[k]);
+    }
+    return m;
+}
+
+// The thread-per-column kernel's interleaved copies (lsq_simt.cu) of a batch:
+// allocated when the build takes it.  Without the memory for them the build
+// runs as it does for small batches
+struct SimtCopies {
+    double *kev = nullptr;
+    float *kev32 = nullptr;
+    uint8_t *lrow_t = nullptr;
+    int W = 0;
+    int64_t ell_map = 0;
+    bool on() const { return kev != nullptr; }
+    void alloc(Scratch &sc, int maxcol, int64_t N, int NS, int K, int n, bool shared) {
+        W = simt_width(maxcol);
+        if (!W) return;
+        ell_map = (((int64_t)(shared ? n : N) + 31) / 32) * (32 * W);
+        const size_t ell = (size_t)(ell_map * (shared ? K : 1));
+        lrow_t = sc.get<uint8_t>(((size_t)NS + 31) / 32 * 32 * kLTile);
+        kev32 = sc.get<float>(ell);
+        if (lrow_t && kev32) kev = sc.get<double>(ell);
+    }
+    cudaError_t values(sam_handle h, int64_t N, int K, int n, bool shared, const int32_t *kcp, int64_t map_nnz,
+                       const double *kcv) const {
+        return simt_values(h, shared ? n : (int)N, shared ? K : 1, W, kcp, map_nnz, kcv, ell_map, kev, kev32);
+    }
+    void args(LsqArgs &a) const {
+        a.kev = kev;
+        a.kev32 = kev32;
+        a.lrow_t = lrow_t;
+        a.ell_map = ell_map;
+        a.ell_w = W;
+    }
+};
+// columns from which a refined FP32 build goes to the thread-per-column kernel
+// and the most unknowns per column on average (its copies pay only where
+// nearly every column is in its size classes)
+constexpr int64_t kSimtMinColumns = 1 << 15, kSimtMeanUnknowns = 9;
+
 sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_0, int NT, const sam_pattern *S,
                       int precision, int refine_steps, const int64_t *M_offsets, int32_t *M_row_ptr,
                       int32_t *M_col_idx, double *M_val, int32_t *col_status, double *res2, double *fro) {
@@ -1375,13 +1424,16 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     if (sg.failed) return SAM_ERR_OOM;
     bool ksym = true, zsym = true;  // structurally symmetric sources / targets
     bool one_structure = false;     // every source, every target: one structure each
+    int maxcol = -1;                // the sources' longest column, -1: not known
     {
         std::vector<DevCsr> all(ak);
         all.insert(all.end(), zs.begin(), zs.end());
         std::vector<char> symv, same;
+        std::vector<int32_t> mrow;
         const std::vector<std::pair<int, int>> ranges{{0, K}, {K, K + NT}};
-        sam_status s = validate_all(h, sc, all, &symv, K > 1 ? &ranges : nullptr, &same);
+        sam_status s = validate_all(h, sc, all, &symv, K > 1 ? &ranges : nullptr, &same, &mrow);
         if (s != SAM_OK) return s;
+        maxcol = longest_column(symv, mrow, K);
         for (size_t q = 0; q < symv.size(); ++q) (q < ak.size() ? ksym : zsym) &= symv[q] != 0;
         one_structure = K > 1 && same[0] && same[1];
     }
@@ -1438,6 +1490,10 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     uint8_t *zloc = sc.get<uint8_t>((size_t)N * kZCap);
     if (!ish || !icnt || !bin || !work || !bin_off || !d_st || !d_r2 || !lrow || !zloc)
         return SAM_ERR_OOM;
+    SimtCopies simt;
+    if (precision == SAM_FP32_REFINE && refine_steps != 0 && h->tape_mode != kTapeRecord && N >= kSimtMinColumns &&
+        total_nnz <= kSimtMeanUnknowns * N)
+        simt.alloc(sc, maxcol, N, NS, K, n, shared);
     // shadow rows, size classes, work list
     ShadowTarget tg;
     tg.zcp = zcp;
@@ -1445,7 +1501,8 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     tg.zbig = NT > 1 ? 1 : 0;
     tg.n = n;
     tg.zloc = zloc;
-    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess)
+    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess ||
+        (simt.on() && simt_rows(h, NS, simt.W, kcp, g->jcp, g->jri, bin, lrow, simt.lrow_t) != cudaSuccess))
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, d_st) != cudaSuccess))
@@ -1469,7 +1526,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         }
     } ev_guard{ev_bins};
     const int32_t *off0 = nullptr;
-    if ((shared ? interleaved_work_list(h, sc, K, n, bin, work, bin_off, &chunks, &off0)
+    if ((shared ? interleaved_work_list(h, sc, K, n, bin, work, bin_off, &chunks, &off0, simt.on())
                 : build_work_list(h, (int)N, bin, work, bin_off)) != cudaSuccess)
         return SAM_ERR_CUDA;
     if (h->record_hist &&
@@ -1501,8 +1558,10 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         if (round_to_f32(h, kn, kcv, kcv32) != cudaSuccess || round_to_f32(h, zn, zcv, zcv32) != cudaSuccess)
             return SAM_ERR_CUDA;
     }
+    if (simt.on() && simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess) return SAM_ERR_CUDA;
     LsqArgs a;
     memset(&a, 0, sizeof(a));
+    if (simt.on()) simt.args(a);
     a.kcv32 = kcv32;
     a.zcv32 = zcv32;
     a.n = n;
@@ -2440,13 +2499,16 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     for (int k = 0; k < K; ++k) ak[k] = DevCsr{A_k[k].n, A_k[k].nnz, A_k[k].row_ptr, A_k[k].col_idx, A_k[k].val};
     bool ksym = true, zsym = true;  // structurally symmetric sources / targets
     bool one_structure = false;     // every source, every target: one structure each
+    int maxcol = -1;                // the sources' longest column, -1: not known
     {
         std::vector<DevCsr> all(ak);
         all.insert(all.end(), zs.begin(), zs.end());
         std::vector<char> symv, same;
+        std::vector<int32_t> mrow;
         const std::vector<std::pair<int, int>> ranges{{0, K}, {K, K + NT}};
-        sam_status s = validate_all(h, tmp, all, &symv, K > 1 ? &ranges : nullptr, &same);
+        sam_status s = validate_all(h, tmp, all, &symv, K > 1 ? &ranges : nullptr, &same, &mrow);
         if (s != SAM_OK) return s;
+        maxcol = longest_column(symv, mrow, K);
         for (size_t q = 0; q < symv.size(); ++q) (q < ak.size() ? ksym : zsym) &= symv[q] != 0;
         one_structure = K > 1 && same[0] && same[1];
     }
@@ -2527,18 +2589,22 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     cudaMemcpyAsync(d_zptr, zptr.data(), sizeof(double *) * NT, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_koff, koff.data(), sizeof(int64_t) * (K + 1), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_zoff, zoff.data(), sizeof(int64_t) * (NT + 1), cudaMemcpyHostToDevice, st);
+    SimtCopies simt;
+    if (precision == SAM_FP32_REFINE && refine_steps != 0 && N >= kSimtMinColumns && total_nnz <= kSimtMeanUnknowns * N)
+        simt.alloc(keep, maxcol, N, NS, K, n, shared);
     ShadowTarget tg;
     tg.zcp = zcp;
     tg.zri = zri;
     tg.zbig = NT > 1 ? 1 : 0;
     tg.n = n;
     tg.zloc = zloc;
-    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess)
+    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess ||
+        (simt.on() && simt_rows(h, NS, simt.W, kcp, g->jcp, g->jri, bin, lrow, simt.lrow_t) != cudaSuccess))
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, d_st) != cudaSuccess))
         return SAM_ERR_CUDA;
-    if ((shared ? interleaved_work_list(h, tmp, K, n, bin, work, bin_off)
+    if ((shared ? interleaved_work_list(h, tmp, K, n, bin, work, bin_off, nullptr, nullptr, simt.on())
                 : build_work_list(h, (int)N, bin, work, bin_off)) != cudaSuccess ||
         split_map_structure(h, K, n, g->mrp, g->mci, M_row_ptr, M_col_idx) != cudaSuccess)
         return SAM_ERR_CUDA;
@@ -2548,6 +2614,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     // ---- value-dependent steps, captured once on a private stream
     LsqArgs a;
     memset(&a, 0, sizeof(a));
+    if (simt.on()) simt.args(a);
     a.kcv32 = kcv32;
     a.zcv32 = zcv32;
     a.n = n;
@@ -2586,6 +2653,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
         // the shadow status of each column is kept in d_st; the solve overwrites it per column
         bool ok = gather_values(h, kn, K, d_koff, d_kptr, kperm, kcv, kcv32) == cudaSuccess &&
                   gather_values(h, zn, NT, d_zoff, d_zptr, zperm, zcv, zcv32) == cudaSuccess &&
+                  (!simt.on() || simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) == cudaSuccess) &&
                   cudaMemsetAsync(M_val, 0, sizeof(double) * (size_t)total_nnz, cs) == cudaSuccess &&
                   cudaMemsetAsync(d_r2, 0, sizeof(double) * (size_t)N, cs) == cudaSuccess &&
                   (!autoref || cudaMemsetAsync(refine_used, 0, (size_t)N, cs) == cudaSuccess) &&

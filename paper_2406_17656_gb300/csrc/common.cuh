@@ -33,6 +33,11 @@ constexpr int kBigJCap = 128;                  // max |J_j|
 constexpr int kBigICap = 1024;                 // max |I_j|
 constexpr int kBigLCap = 16384;                // max stored entries of B_j
 constexpr int kBigTileDoubles = 23 * 1024;     // max |I_j| (|J_j| + 1) (184 KB)
+// lsq_simt.cu's interleaved copies: the most entries of a source column, and
+// bytes per map column in the local rows' copy
+constexpr int kEllW = 12;
+constexpr int kSimtBins = 2, kSimtJ = 9;  // its size classes (0 and 1) and their most unknowns
+constexpr int kLTile = kSimtJ * kEllW;
 constexpr int kZCap = 32;    // target entries per column with a precomputed local row (zloc)
 constexpr int kZOutside = 255;  // zloc value of a target entry outside the shadow rows
 constexpr int kBinNone = 255;
@@ -104,6 +109,12 @@ struct LsqArgs {
     int32_t *colstat;            // per-column status
     const int32_t *work;         // columns grouped by size class
     const int32_t *bin_off;      // [kNumBins+1] offsets into work
+    // interleaved copies for the thread-per-column kernel (lsq_simt.cu), or null
+    const double *kev;
+    const float *kev32;
+    const uint8_t *lrow_t;
+    int64_t ell_map;             // elements of one map in kev / kev32 (shadow_shared)
+    int ell_w;                   // entries kept per source column (simt_width)
     int item_lo, item_hi;        // item_hi > 0: only items [item_lo, item_hi) of the launched class
     int refine_steps;            // < 0: automatic (up to kAutoSteps, FP64 fallback)
     uint8_t *refine_used;        // automatic mode: steps taken per column, kAutoSteps+1 = FP64 fallback
@@ -238,6 +249,21 @@ cudaError_t launch_lsq(sam_handle h, int precision, const LsqArgs &args);
 cudaError_t launch_lsq_big(sam_handle h, const LsqArgs &args, int bin, bool profile = true, bool fp32 = false);
 // one size class (the items args.item_lo/item_hi select, else all of it)
 cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int bin);
+// FP32 + refinement with a thread per column (lsq_simt.cu): size classes whose
+// LsqArgs carry the interleaved copies (kev, kev32, lrow_t)
+cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin);
+// The copies of lsq_simt.cu.  Values: entry u < W of column c of map k (CSC
+// order: cv[kcp[c] + u + k map_nnz]; 0 past the column's end) at
+// ((c >> 5) W + u) 32 + (c & 31) plus k ell_map, for the n columns of the
+// structure of each of K maps
+cudaError_t simt_values(sam_handle h, int n, int K, int W, const int32_t *kcp, int64_t map_nnz, const double *cv,
+                        int64_t ell_map, double *kev, float *kev32);
+// Local rows: of entry u < W of the c-th source column of map column j (its
+// lrow, or the padding row of its size class) at ((j >> 5) kLTile + c W + u) 32 + (j & 31)
+cudaError_t simt_rows(sam_handle h, int n, int W, const int32_t *kcp, const int32_t *jcp, const int32_t *jri,
+                      const uint8_t *bin, const uint8_t *lrow, uint8_t *lrow_t);
+// the width W for sources whose longest column is maxcol; 0: not taken
+int simt_width(int maxcol);
 // the FP64 register tiles of size classes 0-4 (lsq_fp64.cu)
 cudaError_t launch_lsq_fp64_bin(sam_handle h, const LsqArgs &args, int bin);
 cudaError_t launch_adjoint(sam_handle h, int precision, const LsqArgs &args);
