@@ -1595,7 +1595,9 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         a.refine_used = sc.get<uint8_t>((size_t)N);
         work2 = sc.get<int32_t>((size_t)N);
         bin_off2 = sc.get<int32_t>(2);
-        if (!a.refine_used || !work2 || !bin_off2) return SAM_ERR_OOM;
+        a.dense_list = sc.get<int32_t>((size_t)N);
+        a.dense_off = sc.get<int32_t>(2);
+        if (!a.refine_used || !work2 || !bin_off2 || !a.dense_list || !a.dense_off) return SAM_ERR_OOM;
         cudaMemsetAsync(a.refine_used, 0, (size_t)N, st);
     }
     if (autoref) {
@@ -2556,7 +2558,9 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     uint8_t *refine_used = autoref ? keep.get<uint8_t>((size_t)N) : nullptr;
     int32_t *work2 = autoref ? keep.get<int32_t>((size_t)N) : nullptr;
     int32_t *bin_off2 = autoref ? keep.get<int32_t>(kNumBins + 1) : nullptr;
-    if (autoref && (!refine_used || !work2 || !bin_off2)) return SAM_ERR_OOM;
+    int32_t *dense_list = autoref ? keep.get<int32_t>((size_t)N) : nullptr;
+    int32_t *dense_off = autoref ? keep.get<int32_t>(2) : nullptr;
+    if (autoref && (!refine_used || !work2 || !bin_off2 || !dense_list || !dense_off)) return SAM_ERR_OOM;
     // automatic refinement: the two-step launch's own lists (the first
     // launch's work list is read again at every replay)
     RedoLists redo;
@@ -2642,6 +2646,8 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     a.bin_off = bin_off;
     a.refine_steps = refine_steps;
     a.refine_used = refine_used;
+    a.dense_list = dense_list;
+    a.dense_off = dense_off;
     cudaStream_t cs = nullptr;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return SAM_ERR_CUDA;
     const bool prof = h->profiling;

@@ -115,6 +115,10 @@ struct LsqArgs {
     const uint8_t *lrow_t;
     int64_t ell_map;             // elements of one map in kev / kev32 (shadow_shared)
     int ell_w;                   // entries kept per source column (simt_width)
+    // the large class of refined FP32 builds (lsq_dense.cu), or null: the columns
+    // left to its second launch (int32[N]) and their number as a work-list range
+    // (int32[2])
+    int32_t *dense_list, *dense_off;
     int item_lo, item_hi;        // item_hi > 0: only items [item_lo, item_hi) of the launched class
     int refine_steps;            // < 0: automatic (up to kAutoSteps, FP64 fallback)
     uint8_t *refine_used;        // automatic mode: steps taken per column, kAutoSteps+1 = FP64 fallback
@@ -264,6 +268,9 @@ cudaError_t simt_rows(sam_handle h, int n, int W, const int32_t *kcp, const int3
                       const uint8_t *bin, const uint8_t *lrow, uint8_t *lrow_t);
 // the width W for sources whose longest column is maxcol; 0: not taken
 int simt_width(int maxcol);
+// the large class by a Cholesky factor of the normal equations (lsq_dense.cu):
+// refined FP32 builds
+cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin);
 // the FP64 register tiles of size classes 0-4 (lsq_fp64.cu)
 cudaError_t launch_lsq_fp64_bin(sam_handle h, const LsqArgs &args, int bin);
 cudaError_t launch_adjoint(sam_handle h, int precision, const LsqArgs &args);

@@ -7,6 +7,8 @@
 namespace sam {
 
 cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int bin) {
+    if (bin == kBinBig && precision == SAM_FP32_REFINE && args.refine_steps != 0 && args.dense_list)
+        return launch_lsq_dense(h, args, bin);
     if (bin == kBinBig) return launch_lsq_big(h, args, bin, true, precision == SAM_FP32_REFINE);
     if (precision == SAM_FP64) return launch_lsq_fp64_bin(h, args, bin);
     // FP32 tiles: the shape of each size class comes from the handle (sam_tune)
