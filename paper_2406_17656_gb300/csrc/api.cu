@@ -1594,11 +1594,14 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     if (guarded) {
         a.refine_used = sc.get<uint8_t>((size_t)N);
         work2 = sc.get<int32_t>((size_t)N);
-        bin_off2 = sc.get<int32_t>(2);
-        a.dense_list = sc.get<int32_t>((size_t)N);
-        a.dense_off = sc.get<int32_t>(2);
+        a.dense_list = sc.get<int32_t>(2 * (size_t)N);
+        // the counters of the large class's and the re-solve's lists, cleared together
+        a.dense_off = sc.get<int32_t>(6);
+        a.dense_cap = N;
+        bin_off2 = a.dense_off ? a.dense_off + 4 : nullptr;
         if (!a.refine_used || !work2 || !bin_off2 || !a.dense_list || !a.dense_off) return SAM_ERR_OOM;
         cudaMemsetAsync(a.refine_used, 0, (size_t)N, st);
+        cudaMemsetAsync(a.dense_off, 0, sizeof(int32_t) * 6, st);
     }
     if (autoref) {
         // columns that ask for a second step are solved again by a launch of their own
@@ -2557,9 +2560,9 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     const bool autoref = precision == SAM_FP32_REFINE && refine_steps != 0;
     uint8_t *refine_used = autoref ? keep.get<uint8_t>((size_t)N) : nullptr;
     int32_t *work2 = autoref ? keep.get<int32_t>((size_t)N) : nullptr;
-    int32_t *bin_off2 = autoref ? keep.get<int32_t>(kNumBins + 1) : nullptr;
-    int32_t *dense_list = autoref ? keep.get<int32_t>((size_t)N) : nullptr;
-    int32_t *dense_off = autoref ? keep.get<int32_t>(2) : nullptr;
+    int32_t *dense_list = autoref ? keep.get<int32_t>(2 * (size_t)N) : nullptr;
+    int32_t *dense_off = autoref ? keep.get<int32_t>(6) : nullptr;
+    int32_t *bin_off2 = dense_off ? dense_off + 4 : nullptr;  // cleared with them
     if (autoref && (!refine_used || !work2 || !bin_off2 || !dense_list || !dense_off)) return SAM_ERR_OOM;
     // automatic refinement: the two-step launch's own lists (the first
     // launch's work list is read again at every replay)
@@ -2648,6 +2651,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     a.refine_used = refine_used;
     a.dense_list = dense_list;
     a.dense_off = dense_off;
+    a.dense_cap = N;
     cudaStream_t cs = nullptr;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return SAM_ERR_CUDA;
     const bool prof = h->profiling;
@@ -2662,7 +2666,8 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
                   (!simt.on() || simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) == cudaSuccess) &&
                   cudaMemsetAsync(M_val, 0, sizeof(double) * (size_t)total_nnz, cs) == cudaSuccess &&
                   cudaMemsetAsync(d_r2, 0, sizeof(double) * (size_t)N, cs) == cudaSuccess &&
-                  (!autoref || cudaMemsetAsync(refine_used, 0, (size_t)N, cs) == cudaSuccess) &&
+                  (!autoref || (cudaMemsetAsync(refine_used, 0, (size_t)N, cs) == cudaSuccess &&
+                                cudaMemsetAsync(dense_off, 0, sizeof(int32_t) * 6, cs) == cudaSuccess)) &&
                   launch_lsq(h, precision, a) == cudaSuccess &&
                   (!autoref || launch_refine_fallback(h, a, (int)N, work2, bin_off2, h->d_refine, redo) == cudaSuccess) &&
                   status_reduce(h, d_st, N, h->d_flag) == cudaSuccess &&

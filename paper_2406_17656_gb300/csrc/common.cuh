@@ -116,9 +116,10 @@ struct LsqArgs {
     int64_t ell_map;             // elements of one map in kev / kev32 (shadow_shared)
     int ell_w;                   // entries kept per source column (simt_width)
     // the large class of refined FP32 builds (lsq_dense.cu), or null: the columns
-    // left to its second launch (int32[N]) and their number as a work-list range
-    // (int32[2])
+    // left to its second and third launch (int32[2][dense_cap]) and their numbers
+    // as work-list ranges (int32[2][2])
     int32_t *dense_list, *dense_off;
+    int64_t dense_cap;
     int item_lo, item_hi;        // item_hi > 0: only items [item_lo, item_hi) of the launched class
     int refine_steps;            // < 0: automatic (up to kAutoSteps, FP64 fallback)
     uint8_t *refine_used;        // automatic mode: steps taken per column, kAutoSteps+1 = FP64 fallback

@@ -32,41 +32,39 @@ cudaError_t launch_lsq(sam_handle h, int precision, const LsqArgs &args) {
 }
 
 namespace {
-// columns that took s = 1..kAutoSteps steps, and FP64 re-solves: per-thread
-// counts, summed over the warp by shuffles, one shared atomic per warp
-__global__ void refine_count_kernel(int64_t N, const uint8_t *used, unsigned long long *counts) {
-    __shared__ unsigned long long sh[kAutoSteps + 1];
-    if (threadIdx.x <= kAutoSteps) sh[threadIdx.x] = 0ull;
+// the columns flagged for the FP64 re-solve, in any order, into list;
+// off[1] receives their number (off[0] = 0: the list as a work-list range);
+// counts (nullable): the columns that took s = 1..kAutoSteps steps, and the
+// FP64 re-solves (per-thread counts, one shared atomic per warp)
+__global__ void __launch_bounds__(256) flag_list_kernel(int N, const int32_t *colstat, const uint8_t *used, int32_t *list,
+                                                        int32_t *off, unsigned long long *counts) {
+    __shared__ unsigned sh[kAutoSteps + 1];
+    if (threadIdx.x <= kAutoSteps) sh[threadIdx.x] = 0u;
     __syncthreads();
+    const int lane = threadIdx.x & 31;
     unsigned c[kAutoSteps + 1] = {};
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
-        const int u = used[j];
+    for (int64_t j0 = (int64_t)blockIdx.x * 256; j0 < N; j0 += (int64_t)gridDim.x * 256) {
+        const int64_t j = j0 + threadIdx.x;
+        const bool f = j < N && colstat[j] == kStRefine;
+        const int u = counts && j < N ? used[j] : 0;
 #pragma unroll
         for (int v = 0; v <= kAutoSteps; ++v) c[v] += (u == v + 1) ? 1u : 0u;
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (!m) continue;
+        const int leader = __ffs(m) - 1;
+        int base = 0;
+        if (lane == leader) base = atomicAdd(&off[1], __popc(m));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (f) list[base + __popc(m & ((1u << lane) - 1u))] = (int)j;
     }
+    if (!counts) return;
 #pragma unroll
     for (int v = 0; v <= kAutoSteps; ++v) {
-        unsigned t = c[v];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&sh[v], (unsigned long long)t);
+        const unsigned t = __reduce_add_sync(0xffffffffu, c[v]);
+        if (lane == 0 && t) atomicAdd(&sh[v], t);
     }
     __syncthreads();
-    if (threadIdx.x <= kAutoSteps && sh[threadIdx.x]) atomicAdd(&counts[threadIdx.x], sh[threadIdx.x]);
-}
-
-// the columns flagged for the FP64 re-solve, in any order, into list;
-// off[1] receives their number (off[0] = 0: the list as a work-list range)
-__global__ void flag_list_kernel(int N, const int32_t *colstat, int32_t *list, int32_t *off) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool f = j < N && colstat[j] == kStRefine;
-    const unsigned m = __ballot_sync(0xffffffffu, f);
-    if (!m) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(&off[1], __popc(m));
-    base = __shfl_sync(m, base, leader);
-    if (f) list[base + __popc(m & ((1u << lane) - 1u))] = j;
+    if (threadIdx.x <= kAutoSteps && sh[threadIdx.x]) atomicAdd(&counts[threadIdx.x], (unsigned long long)sh[threadIdx.x]);
 }
 }  // namespace
 
@@ -92,9 +90,13 @@ cudaError_t launch_refine_fallback(sam_handle h, const LsqArgs &args, int N, int
         for (int b = 0; b < kBinBig; ++b)
             if ((e = launch_lsq_bin(h, SAM_FP32_REFINE, a2, b)) != cudaSuccess) return e;
     }
-    if ((e = cudaMemsetAsync(list_off, 0, sizeof(int32_t) * 2, st)) != cudaSuccess) return e;
+    // (list_off is zero: cleared with the batch's other counters)
+    if (counts && (e = cudaMemsetAsync(counts, 0, sizeof(int64_t) * (kAutoSteps + 1), st)) != cudaSuccess) return e;
     if (N > 0) {
-        flag_list_kernel<<<(N + 255) / 256, 256, 0, st>>>(N, args.colstat, list, list_off);
+        int blocks = (N + 255) / 256;
+        if (blocks > handle_sms(h) * 8) blocks = handle_sms(h) * 8;
+        flag_list_kernel<<<blocks, 256, 0, st>>>(N, args.colstat, args.refine_used, list, list_off,
+                                                 reinterpret_cast<unsigned long long *>(counts));
         count_launch(h);
     }
     // every flagged column, whatever its size class, by the FP64 kernel of
@@ -104,14 +106,6 @@ cudaError_t launch_refine_fallback(sam_handle h, const LsqArgs &args, int N, int
     a.bin_off = list_off;
     a.item_lo = a.item_hi = 0;
     if ((e = launch_lsq_big(h, a, 0, false)) != cudaSuccess) return e;
-    if (counts) {
-        if ((e = cudaMemsetAsync(counts, 0, sizeof(int64_t) * (kAutoSteps + 1), st)) != cudaSuccess) return e;
-        int blocks = (N + 255) / 256;
-        if (blocks > handle_sms(h) * 4) blocks = handle_sms(h) * 4;
-        if (blocks < 1) blocks = 1;
-        refine_count_kernel<<<blocks, 256, 0, st>>>(N, args.refine_used, reinterpret_cast<unsigned long long *>(counts));
-        count_launch(h);
-    }
     return cudaGetLastError();
 }
 

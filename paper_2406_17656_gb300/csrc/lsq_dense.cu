@@ -10,6 +10,18 @@
 // (lsq_big.cu) the dense work drops from 2 n^2 (m - n / 3) to about
 // nnz(B) n / 2 + n^3 / 6 multiply-adds, since G's rows are sums over the stored
 // entries of B alone, and no reflector waits for another's norm.
+//
+// Where the time goes (clock64 timers in an instrumented copy, 81 x 49 columns of
+// Q1 level-3 maps, seven blocks per SM): factorisation 28%, triangular solves 16%,
+// row index and scatter 16%, Gram matrix 9%, the FP64 passes 14%.  The
+// factorisation is one warp's for up to 52 unknowns: a 4-warp tile with a
+// block barrier per pivot issued 480 warp instructions per pivot against 90.
+// Shared memory decides the blocks per SM: the dense FP32 rows of [B c] live
+// only until G exists, then the row lists and B's FP64 values take their place.
+// 128 threads per small block: 96 cost 1%, 64 cost 23%.
+//
+// Measured: Q1 256^2, 2 maps, level 3, the whole call: 60.1 -> 8.7 ms; 7,700
+// columns of up to 201 x 96 with 7,300 entries, 2 maps: 47.8 -> 15.3 ms.
 #include <cfloat>
 #include <climits>
 
@@ -27,15 +39,15 @@ __device__ __forceinline__ V wsum(V v) {
     return v;
 }
 
+template <int MAXJ>
 struct __align__(16) DenseHdr {
-    long long colA[kBigJCap];     // value offset of column c of B (this map's values)
-    int kcol[kBigJCap];           // structure offset of column c
-    unsigned short cb[kBigJCap + 2];  // first entry of column c in gather order
-    float colk[kBigJCap + 4];     // column k of L during the factorisation
-    float inv[kBigJCap];          // 1 / L_kk
-    float g[kBigJCap];            // B^T r, then the correction
-    double x[kBigJCap];           // the vector of the next product B x
-    double m[kBigJCap];           // the solution
+    long long colA[MAXJ];     // value offset of column c of B (this map's values)
+    int kcol[MAXJ];           // structure offset of column c
+    unsigned short cb[MAXJ + 2];  // first entry of column c in gather order
+    float inv[MAXJ];          // 1 / L_kk
+    float g[MAXJ];            // B^T r, then the correction
+    double x[MAXJ];           // the vector of the next product B x
+    double m[MAXJ];           // the solution
     double part[32];              // partial sums of the warps
     int scan[32];
     int status, nB, lo, hi, nI, brk, redo, fallback;
@@ -52,11 +64,11 @@ struct DenseLayout {
     double *r;               // c, then the residual [nI]
     unsigned short *rowstart;  // [nI + 1]
     unsigned short *row;     // local row of every entry, by columns [nB]
-    unsigned short *pl;      // entries by rows: their index by columns [nB]
-    unsigned char *cl;       // and their column [nB]
     float *L;                // rows 0..n of [G b], then of L, packed
-    float *B;                // [B c] dense, rows of ldb floats, until G is formed
-    double *val;             // then B's entries by columns [nB], when they fit there
+    float *B;                // [B c] dense, rows of ldb floats, until G is formed; then there
+    unsigned short *pl;      // the entries by rows: their index by columns [nB]
+    unsigned char *cl;       // their column [nB]
+    double *val;             // and, when there is room (vals), B's entries by columns [nB]
     bool vals;
     __device__ size_t set(unsigned char *base, int nI_, int n_, int nB_, int words_, size_t room) {
         nI = nI_, n = n_, nB = nB_, words = words_;
@@ -69,31 +81,120 @@ struct DenseLayout {
             return p;
         };
         r = (double *)take(sizeof(double) * nI);
-        const size_t dense = sizeof(float) * (size_t)nI * ldb, all = sizeof(double) * (size_t)nB;
-        B = (float *)take(all > dense && all <= room ? all : dense);
-        val = (double *)B;
-        vals = all <= room || all <= dense;
+        const size_t dense = sizeof(float) * (size_t)nI * ldb, v8 = sizeof(double) * (size_t)nB;
+        const size_t lists = ((3 * (size_t)nB + 15) & ~(size_t)15), all = v8 + lists;
+        vals = all <= (dense > room ? dense : room);
+        const size_t need = vals ? all : lists;
+        unsigned char *u = take(need > dense ? need : dense);
+        B = (float *)u;
+        pl = (unsigned short *)u;
+        cl = u + 2 * nB;
+        val = (double *)(u + lists);
         L = (float *)take(sizeof(float) * tri(n + 1));
         bm = (unsigned *)take(sizeof(unsigned) * words);
         pre = (unsigned short *)take(sizeof(unsigned short) * words);
         mask = (unsigned *)take(sizeof(unsigned) * nI * nw);
         rowstart = (unsigned short *)take(sizeof(unsigned short) * (nI + 1));
         row = (unsigned short *)take(sizeof(unsigned short) * nB);
-        pl = (unsigned short *)take(sizeof(unsigned short) * nB);
-        cl = (unsigned char *)take(nB);
         return o;
     }
 };
 
 // One column per block of NT threads.  Columns whose arrays take more than
 // `cap` bytes (or whose rows span too far) are appended to rest for the next kernel.
-template <int NT>
-__global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, unsigned cap, int32_t *rest,
+// Blocks of NT threads, BLOCKS per SM.  The factorisation runs on the first GT
+// threads as a TY x TX grid over RS TY rows (G's and b) and CS TX columns.
+template <int NT_, int BLOCKS_, int GT_, int TX_, int RS_, int CS_>
+struct DenseShape {
+    static constexpr int NT = NT_, BLOCKS = BLOCKS_, GT = GT_, TX = TX_, TY = GT_ / TX_, RS = RS_, CS = CS_;
+    static constexpr int MAXJ = TY * RS - 1 < TX * CS ? TY * RS - 1 : TX * CS;
+    static constexpr int XS = (MAXJ + 31) / 32;  // unknowns per lane in the solves
+    // the pivot column in shared memory, once by rows and once by columns: a
+    // thread's values are contiguous (padded to whole 16-byte chunks)
+    static constexpr int RP = (RS + 3) & ~3, CP = (CS + 3) & ~3, UW = TY * RP + TX * CP;
+};
+using DenseSmall = DenseShape<128, 7, 32, 4, 7, 13>;   // up to 52 unknowns
+using DenseMedium = DenseShape<128, 3, 128, 8, 9, 16>;  // up to 128
+using DenseLarge = DenseShape<512, 1, 128, 8, 9, 16>;  // up to 128
+static_assert(DenseSmall::UW % 4 == 0 && DenseLarge::UW % 4 == 0, "alignment");
+static_assert(DenseSmall::MAXJ == 52 && DenseLarge::MAXJ == kBigJCap, "shapes");
+
+// the threads of the factorisation (named barrier 1 when they are several warps)
+template <class SH>
+__device__ __forceinline__ void group_sync() {
+    if constexpr (SH::GT == 32) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"n"(SH::GT) : "memory");
+}
+
+struct Pivots {
+    float dmax, dmin;
+    bool brk;
+    int status;
+};
+
+// Pivots k = TX T0 .. TX T0 + TX - 1 and on: right-looking, thread (ty, tx)
+// holding rows ty + TY q of columns tx + TX t (the blocks that reach the
+// lower triangle).  The pivot column goes unscaled through ub (double-buffered),
+// one barrier per pivot; row n is b.  Elements past row or column n are never
+// used, so nothing tests for them; a finished column keeps its unscaled values.
+template <class SH, int T0>
+__device__ __forceinline__ void factor_from(float (&a)[SH::RS][SH::CS], float *ub, float *invs, int n, int tx, int ty,
+                                            Pivots &pv) {
+    constexpr int TX = SH::TX, TY = SH::TY, RS = SH::RS, CS = SH::CS, RP = SH::RP, CP = SH::CP, Q0 = TX * T0 / TY;
+    if constexpr (T0 < CS) {
+        if (TX * T0 >= n) return;
+        for (int kk = 0; kk < TX; ++kk) {
+            const int k = TX * T0 + kk;
+            if (k >= n) return;
+            float *ur = ub + (k & 1) * SH::UW, *uc = ur + TY * RP;
+            if (tx == kk) {
+#pragma unroll
+                for (int q = Q0; q < RS; ++q) {
+                    const int i = ty + TY * q;
+                    ur[ty * RP + q] = a[q][T0];
+                    if (i < TX * CS) uc[(i % TX) * CP + i / TX] = a[q][T0];
+                }
+            }
+            group_sync<SH>();
+            const float d = uc[kk * CP + T0];
+            if (!pv.brk && !(fabsf(d) <= FLT_MAX)) pv.status = kStNonfinite;  // (past a breakdown every pivot is NaN)
+            pv.brk = pv.brk || !(d > 0.f);
+            pv.dmax = fmaxf(pv.dmax, d);
+            pv.dmin = fminf(pv.dmin, d);
+            const float inv = rsqrtf(d), ninv2 = -inv * inv;
+            if (tx == kk && ty == 0) invs[k] = inv;
+            float ui[RP], uj[CP];
+#pragma unroll
+            for (int q = Q0 / 4; q < RP / 4; ++q) *reinterpret_cast<float4 *>(ui + 4 * q) = *reinterpret_cast<const float4 *>(ur + ty * RP + 4 * q);
+#pragma unroll
+            for (int t = T0 / 4; t < CP / 4; ++t) *reinterpret_cast<float4 *>(uj + 4 * t) = *reinterpret_cast<const float4 *>(uc + tx * CP + 4 * t);
+#pragma unroll
+            for (int q = Q0; q < RS; ++q) ui[q] *= ninv2;
+            // (rows and columns up to k keep their values)
+            if (ty + TY * Q0 <= k) ui[Q0] = 0.f;
+            if constexpr (Q0 + 1 < RS && TY < TX) {
+                if (ty + TY * (Q0 + 1) <= k) ui[Q0 + 1] = 0.f;
+            }
+            if (tx <= kk) uj[T0] = 0.f;
+#pragma unroll
+            for (int t = T0; t < CS; ++t)
+#pragma unroll
+                for (int q = Q0; q < RS; ++q)
+                    if (TY * q + TY - 1 >= TX * t) a[q][t] = fmaf(ui[q], uj[t], a[q][t]);
+        }
+        factor_from<SH, T0 + 1>(a, ub, invs, n, tx, ty, pv);
+    }
+}
+
+template <class SH>
+__global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs args, int bin, unsigned cap, int32_t *rest,
                                                        int32_t *rest_off) {
-    constexpr int NW = NT / 32;
+    constexpr int NT = SH::NT, NW = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DenseHdr &H = *reinterpret_cast<DenseHdr *>(smem_raw);
-    unsigned char *base = smem_raw + sizeof(DenseHdr);
+    using Hdr = DenseHdr<SH::MAXJ>;
+    Hdr &H = *reinterpret_cast<Hdr *>(smem_raw);
+    float *ub = reinterpret_cast<float *>(smem_raw + sizeof(Hdr));  // the factorisation's pivot column
+    unsigned char *base = smem_raw + sizeof(Hdr) + 8 * SH::UW;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     const int w0 = args.bin_off[bin] + (args.item_hi > 0 ? args.item_lo : 0);
@@ -129,7 +230,7 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
             for (int c0 = 0; c0 < n; c0 += 32) {
                 const int c = c0 + lane;
                 int len = 0;
-                if (c < n && n <= kBigJCap) {
+                if (c < n && n <= SH::MAXJ) {
                     const int col = args.jri[jb + c];
                     const int a0 = args.kcp[col];
                     len = args.kcp[col + 1] - a0;
@@ -146,7 +247,7 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
                     const int y = __shfl_up_sync(0xffffffffu, incl, o);
                     if (lane >= o) incl += y;
                 }
-                if (c < n && n <= kBigJCap) H.cb[c + 1] = (unsigned short)min(run + incl, 65535);
+                if (c < n && n <= SH::MAXJ) H.cb[c + 1] = (unsigned short)min(run + incl, 65535);
                 run += __shfl_sync(0xffffffffu, incl, 31);
             }
             lo = __reduce_min_sync(0xffffffffu, lo);
@@ -165,7 +266,7 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
         const int64_t span = (int64_t)H.hi - lo + 1;
         const int words = (int)((span + 31) >> 5);
         DenseLayout D;
-        bool take = n <= kBigJCap && nI >= n && nI <= kBigICap && nB <= kBigLCap && words <= (int)cap;
+        bool take = n <= SH::MAXJ && nI >= n && nI <= kBigICap && nB <= kBigLCap && words <= (int)cap;
         if (take) {
             // the values stay in shared memory when there is room for them
             const size_t least = D.set(base, nI, n, nB, words, 0);
@@ -305,76 +406,104 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
             }
         }
         // ---- G = L L^T; the row of b becomes y = L^{-1} b
-        float dmax = 0.f, dmin = FLT_MAX;
-        bool brk = false;
-        for (int k = 0; k < n; ++k) {
-            const float d = D.L[tri(k) + k];
-            if (!brk && !(fabsf(d) <= FLT_MAX) && tid == 0) atomicMax(&H.status, (int)kStNonfinite);
-            brk = brk || !(d > 0.f);
-            dmax = fmaxf(dmax, d);
-            dmin = fminf(dmin, d);
-            const float inv = rsqrtf(d);
-            for (int i = k + 1 + tid; i <= n; i += NT) {
-                const float v = D.L[tri(i) + k] * inv;
-                D.L[tri(i) + k] = v;
-                H.colk[i] = v;
-            }
-            if (tid == 0) H.inv[k] = inv;
-            __syncthreads();
-            float lj[4];
+        __syncthreads();
+        if (tid < SH::GT) {
+            constexpr int TX = SH::TX, TY = SH::TY, RS = SH::RS, CS = SH::CS;
+            const int tx = tid % TX, ty = tid / TX;
+            float a[RS][CS];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int j = k + 1 + lane + 32 * t;
-                lj[t] = j < n ? H.colk[j] : 0.f;
-            }
-            for (int i = k + 1 + warp; i <= n; i += NW) {
-                const float li = H.colk[i];
-                float *Li = D.L + tri(i);
+            for (int q = 0; q < RS; ++q)
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int j = k + 1 + lane + 32 * t;
-                    if (j <= i && j < n) Li[j] = fmaf(-li, lj[t], Li[j]);
+                for (int t = 0; t < CS; ++t) {
+                    const int i = ty + TY * q, j = tx + TX * t;
+                    a[q][t] = TY * q + TY - 1 >= TX * t && i <= n && j <= i && j < n ? D.L[tri(i) + j] : 0.f;
+                }
+            Pivots pv{0.f, FLT_MAX, false, kStOk};
+            factor_from<SH, 0>(a, ub, H.inv, n, tx, ty, pv);
+            group_sync<SH>();
+#pragma unroll
+            for (int t = 0; t < CS; ++t) {
+                const int j = tx + TX * t;
+                const float inv = j < n ? H.inv[j] : 0.f;
+#pragma unroll
+                for (int q = 0; q < RS; ++q) {
+                    const int i = ty + TY * q;
+                    if (TY * q + TY - 1 >= TX * t && i <= n && j < i && j < n) D.L[tri(i) + j] = a[q][t] * inv;
                 }
             }
-            __syncthreads();
+            if (tid == 0) {
+                if (pv.status != kStOk) H.status = max(H.status, pv.status);
+                H.brk = pv.brk ? 1 : 0;
+                H.kap2 = pv.dmax / pv.dmin;  // a lower bound on kappa(B)^2
+            }
+            group_sync<SH>();
         }
-        const float kap2 = dmax / dmin;
-        // triangular solves by warp 0: entries c = lane + 32 t in x[]
-        float x[4];
+        // triangular solves by warp 0: entries c = lane + 32 t in x[].  The
+        // chain of a step is a product, a shuffle and a multiply-add; L's
+        // elements are loaded a step ahead
+        constexpr int XS = SH::XS;
+        float x[XS], iv[XS];
         auto back = [&]() {  // L^T x = y
-            for (int k = n - 1; k >= 0; --k) {
-                const int t0 = k >> 5;
-                float xk = (t0 == 0 ? x[0] : t0 == 1 ? x[1] : t0 == 2 ? x[2] : x[3]) * H.inv[k];
-                xk = __shfl_sync(0xffffffffu, xk, k & 31);
-                const float *Lk = D.L + tri(k);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int c = lane + 32 * t;
-                    if (c < k) x[t] = fmaf(-Lk[c], xk, x[t]);
-                    else if (c == k) x[t] = xk;
+            for (int t0 = XS - 1; t0 >= 0; --t0) {
+                if (32 * t0 >= n) continue;
+                const int kh = min(32 * t0 + 31, n - 1);
+                float l[XS], ln[XS];
+#pragma unroll
+                for (int t = 0; t <= t0; ++t) l[t] = lane + 32 * t < kh ? D.L[tri(kh) + lane + 32 * t] : 0.f;
+#pragma unroll 4
+                for (int k = kh; k >= 32 * t0; --k) {
+                    const int k1 = max(k - 1, 0);
+#pragma unroll
+                    for (int t = 0; t <= t0; ++t) ln[t] = lane + 32 * t < k1 ? D.L[tri(k1) + lane + 32 * t] : 0.f;
+                    const float xk = __shfl_sync(0xffffffffu, x[t0] * iv[t0], k & 31);
+#pragma unroll
+                    for (int t = 0; t <= t0; ++t) {
+                        x[t] = fmaf(-l[t], xk, x[t]);
+                        l[t] = ln[t];
+                    }
                 }
             }
+#pragma unroll
+            for (int t = 0; t < XS; ++t) x[t] *= iv[t];
         };
         auto fwd = [&]() {  // L y = g
-            for (int k = 0; k < n; ++k) {
-                const int t0 = k >> 5;
-                float yk = (t0 == 0 ? x[0] : t0 == 1 ? x[1] : t0 == 2 ? x[2] : x[3]) * H.inv[k];
-                yk = __shfl_sync(0xffffffffu, yk, k & 31);
+            int b[XS];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int c = lane + 32 * t;
-                    if (c > k && c < n) x[t] = fmaf(-D.L[tri(c) + k], yk, x[t]);
-                    else if (c == k) x[t] = yk;
+            for (int t = 0; t < XS; ++t) b[t] = tri(lane + 32 * t);
+#pragma unroll
+            for (int t0 = 0; t0 < XS; ++t0) {
+                if (32 * t0 >= n) continue;
+                const int ke = min(32 * t0 + 32, n);
+                float l[XS], ln[XS];
+                auto load = [&](float (&o)[XS], int k) {
+#pragma unroll
+                    for (int t = t0; t < XS; ++t) o[t] = lane + 32 * t > k && lane + 32 * t < n ? D.L[b[t] + k] : 0.f;
+                };
+                load(l, 32 * t0);
+#pragma unroll 4
+                for (int k = 32 * t0; k < ke; ++k) {
+                    load(ln, k + 1);
+                    const float yk = __shfl_sync(0xffffffffu, x[t0] * iv[t0], k & 31);
+#pragma unroll
+                    for (int t = t0; t < XS; ++t) {
+                        x[t] = fmaf(-l[t], yk, x[t]);
+                        l[t] = ln[t];
+                    }
                 }
             }
+#pragma unroll
+            for (int t = 0; t < XS; ++t) x[t] *= iv[t];
         };
         if (warp == 0) {
             float m2 = 0.f;
 #pragma unroll
-            for (int t = 0; t < 4; ++t) x[t] = lane + 32 * t < n ? D.L[tri(n) + lane + 32 * t] : 0.f;
+            for (int t = 0; t < XS; ++t) iv[t] = lane + 32 * t < n ? H.inv[lane + 32 * t] : 0.f;
+#pragma unroll
+            for (int t = 0; t < XS; ++t) x[t] = lane + 32 * t < n ? D.L[tri(n) + lane + 32 * t] : 0.f;
             back();
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
+            for (int t = 0; t < XS; ++t) {
                 const int c = lane + 32 * t;
                 if (c < n) {
                     H.x[c] = H.m[c] = widen(x[t]);
@@ -384,7 +513,7 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
             m2 = wsum(m2);
             if (lane == 0) {
                 H.msq = m2;
-                H.fallback = brk ? 1 : 0;
+                H.fallback = H.brk;
                 H.redo = 0;
             }
         }
@@ -433,12 +562,12 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
             __syncthreads();
             if (warp == 0) {
 #pragma unroll
-                for (int t = 0; t < 4; ++t) x[t] = lane + 32 * t < n ? H.g[lane + 32 * t] : 0.f;
+                for (int t = 0; t < XS; ++t) x[t] = lane + 32 * t < n ? H.g[lane + 32 * t] : 0.f;
                 fwd();
                 back();
                 float dsq = 0.f, dg = 0.f;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
+                for (int t = 0; t < XS; ++t) {
                     const int c = lane + 32 * t;
                     if (c < n) {
                         H.x[c] = widen(x[t]);
@@ -454,7 +583,7 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
                     const float msq = H.msq;
                     if (step == 0) H.da2 = dsq;
                     const float da2 = H.da2;
-                    const float rk = (float)(kRhoSafety * kU32) * kap2;
+                    const float rk = (float)(kRhoSafety * kU32) * H.kap2;
                     bool miss = !(rk < 0.5f) || rk * rk * dsq > kTol2 * (1.f - rk) * (1.f - rk) * msq;
                     miss = miss || 4.f * kC * kC * da2 >= msq || 4.f * kC * kC * da2 * dsq > kTol2 * msq * msq;
                     if (step > 0 && dsq > (float)kNoise2 * msq) {
@@ -498,14 +627,15 @@ __global__ void __launch_bounds__(NT) lsq_dense_kernel(LsqArgs args, int bin, un
     }
 }
 
-template <int NT>
-cudaError_t launch_dense(sam_handle h, const LsqArgs &a, int bin, int per_sm, int32_t *rest, int32_t *rest_off) {
+template <class SH>
+cudaError_t launch_dense(sam_handle h, const LsqArgs &a, int bin, int32_t *rest, int32_t *rest_off) {
+    constexpr int per_sm = SH::BLOCKS;
     // the shared memory of an SM split over per_sm blocks (1 KB of each is the system's)
     const size_t smem = (size_t)((per_sm == 1 ? 232448 : 233472 / per_sm - 1024) & ~127);
-    auto kern = lsq_dense_kernel<NT>;
+    auto kern = lsq_dense_kernel<SH>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<handle_sms(h) * per_sm, NT, smem, handle_stream(h)>>>(a, bin, (unsigned)(smem - sizeof(DenseHdr)), rest, rest_off);
+    kern<<<handle_sms(h) * per_sm, SH::NT, smem, handle_stream(h)>>>(a, bin, (unsigned)(smem - sizeof(DenseHdr<SH::MAXJ>) - 8 * SH::UW), rest, rest_off);
     count_launch(h);
     return cudaGetLastError();
 }
@@ -513,16 +643,20 @@ cudaError_t launch_dense(sam_handle h, const LsqArgs &a, int bin, int per_sm, in
 }  // namespace
 
 cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
-    // small columns by small blocks, the others by one block per SM
-    cudaError_t e = cudaMemsetAsync(args.dense_off, 0, sizeof(int32_t) * 2, handle_stream(h));
-    if (e != cudaSuccess) return e;
+    // small columns by small blocks, each next launch those that are left
+    cudaError_t e;
+    if (args.item_hi > 0 && (e = cudaMemsetAsync(args.dense_off, 0, sizeof(int32_t) * 4, handle_stream(h))) != cudaSuccess)
+        return e;  // (a chunk of a batch: the counters are used again)
     profile_begin(h, bin);
-    if ((e = launch_dense<128>(h, args, bin, 7, args.dense_list, args.dense_off)) != cudaSuccess) return e;
+    if ((e = launch_dense<DenseSmall>(h, args, bin, args.dense_list, args.dense_off)) != cudaSuccess) return e;
     LsqArgs a = args;
     a.item_lo = a.item_hi = 0;
     a.work = args.dense_list;
     a.bin_off = args.dense_off;
-    if ((e = launch_dense<512>(h, a, 0, 1, nullptr, nullptr)) != cudaSuccess) return e;
+    if ((e = launch_dense<DenseMedium>(h, a, 0, args.dense_list + args.dense_cap, args.dense_off + 2)) != cudaSuccess) return e;
+    a.work = args.dense_list + args.dense_cap;
+    a.bin_off = args.dense_off + 2;
+    if ((e = launch_dense<DenseLarge>(h, a, 0, nullptr, nullptr)) != cudaSuccess) return e;
     profile_end(h, bin);
     return cudaSuccess;
 }
