@@ -83,7 +83,16 @@ __global__ void permute_scatter_kernel(int64_t nnz, const int32_t *perm, const d
 cudaError_t launch_adjoint(sam_handle h, int precision, const LsqArgs &args) {
     cudaError_t e;
     const bool tape = args.fac_mode == kTapeReplay;
-    for (int b = 0; b < kRegBins; ++b) {
+    if (args.kev) {
+        // a thread per column for the smallest classes, then the columns it
+        // leaves by the larger class's QR tile
+        if ((e = launch_adjoint_simt(h, args)) != cudaSuccess) return e;
+        LsqArgs a = args;
+        a.work = args.dense_list;
+        a.bin_off = args.dense_off - (kSimtBins - 1);
+        if ((e = launch_adjoint_f32_bin(h, a, kSimtBins - 1)) != cudaSuccess) return e;
+    }
+    for (int b = args.kev ? kSimtBins : 0; b < kRegBins; ++b) {
         // with a tape the two smallest classes still recompute R: their QR
         // (at most 9 unknowns) costs less than reading and unpacking the tape
         if (tape && b >= 2) e = launch_adjoint_tape_bin(h, precision, args, b);

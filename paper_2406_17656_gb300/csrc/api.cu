@@ -1491,7 +1491,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     if (!ish || !icnt || !bin || !work || !bin_off || !d_st || !d_r2 || !lrow || !zloc)
         return SAM_ERR_OOM;
     SimtCopies simt;
-    if (precision == SAM_FP32_REFINE && refine_steps != 0 && h->tape_mode != kTapeRecord && N >= kSimtMinColumns &&
+    if (precision == SAM_FP32_REFINE && refine_steps != 0 && N >= kSimtMinColumns &&
         total_nnz <= kSimtMeanUnknowns * N)
         simt.alloc(sc, maxcol, N, NS, K, n, shared);
     // shadow rows, size classes, work list
@@ -2031,13 +2031,16 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     if (sg.failed) return SAM_ERR_OOM;
     bool ksym = true, zsym = true;  // structurally symmetric sources / targets
     bool one_structure = false;     // every source, every target: one structure each
+    int maxcol = -1;                // the sources' longest column, -1: not known
     {
         std::vector<DevCsr> all(ak);
         all.insert(all.end(), zs.begin(), zs.end());
         std::vector<char> symv, same;
+        std::vector<int32_t> mrow;
         const std::vector<std::pair<int, int>> ranges{{0, K}, {K, 2 * K}};
-        sam_status s = validate_all(h, sc, all, &symv, K > 1 ? &ranges : nullptr, &same);
+        sam_status s = validate_all(h, sc, all, &symv, K > 1 ? &ranges : nullptr, &same, &mrow);
         if (s != SAM_OK) return s;
+        maxcol = longest_column(symv, mrow, K);
         for (size_t q = 0; q < symv.size(); ++q) (q < ak.size() ? ksym : zsym) &= symv[q] != 0;
         one_structure = K > 1 && same[0] && same[1];
     }
@@ -2073,13 +2076,23 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     if (!ish || !icnt || !bin || !colstat || !nbcnt || !dB_off || !work || !bin_off || !dbase || !dzval ||
         !dak_csc || !lrow || !zloc)
         return SAM_ERR_OOM;
+    SimtCopies simt;
+    int32_t *adj_off = nullptr, *adj_list = nullptr;
+    if (precision == SAM_FP32_REFINE && refine_steps != 0 && N >= kSimtMinColumns && mtot <= kSimtMeanUnknowns * N) {
+        adj_off = sc.get<int32_t>(4);
+        adj_list = sc.get<int32_t>((size_t)N);
+        if (adj_off && adj_list) simt.alloc(sc, maxcol, N, NS, K, n, shared);
+        if (simt.on()) cudaMemsetAsync(adj_off, 0, sizeof(int32_t) * 4, st);
+    }
     ShadowTarget tg;
     tg.zcp = zcp;
     tg.zri = zri;
     tg.zbig = 1;
     tg.n = n;
     tg.zloc = zloc;
-    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, colstat, nbcnt, lrow, tg) != cudaSuccess)
+    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, colstat, nbcnt, lrow, tg) != cudaSuccess ||
+        (simt.on() && (simt_rows(h, NS, simt.W, kcp, g->jcp, g->jri, bin, lrow, simt.lrow_t) != cudaSuccess ||
+                       simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess)))
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, colstat) != cudaSuccess || replicate_cols(h, K, n, nbcnt) != cudaSuccess))
@@ -2142,6 +2155,11 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     a.dmres = d_dmr;
     a.dbase = dbase;
     a.znnz = zn;
+    if (simt.on()) {
+        simt.args(a);
+        a.dense_list = adj_list;
+        a.dense_off = adj_off + 1;
+    }
     if ((s = tape_args(h, sc, g, N, precision, kTapeReplay, a)) != SAM_OK) return s;
     if (launch_adjoint(h, precision, a) != cudaSuccess) return SAM_ERR_CUDA;
     if (adjoint_reduce(h, (int)N, kcp, g->mrp, dbase, dB, dak_csc) != cudaSuccess ||

@@ -115,6 +115,7 @@ struct LsqArgs {
     const uint8_t *lrow_t;
     int64_t ell_map;             // elements of one map in kev / kev32 (shadow_shared)
     int ell_w;                   // entries kept per source column (simt_width)
+    // (the adjoint: the columns the thread-per-column kernel leaves; builds:)
     // the large class of refined FP32 builds (lsq_dense.cu), or null: the columns
     // left to its second and third launch (int32[2][dense_cap]) and their numbers
     // as work-list ranges (int32[2][2])
@@ -257,6 +258,9 @@ cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int
 // FP32 + refinement with a thread per column (lsq_simt.cu): size classes whose
 // LsqArgs carry the interleaved copies (kev, kev32, lrow_t)
 cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin);
+// the adjoint of its size classes; the columns it leaves to the QR kernel go to
+// args.dense_list, their number to args.dense_off[1] (zeroed by the caller)
+cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args);
 // The copies of lsq_simt.cu.  Values: entry u < W of column c of map k (CSC
 // order: cv[kcp[c] + u + k map_nnz]; 0 past the column's end) at
 // ((c >> 5) W + u) 32 + (c & 31) plus k ell_map, for the n columns of the

@@ -42,19 +42,21 @@ namespace {
 constexpr __host__ __device__ int tri(int q) { return q * (q + 1) / 2; }
 
 constexpr int kSimtWarps = 16;  // one-warp blocks per SM at most (128 registers each)
-constexpr int kAhead = 1;       // columns loaded ahead of their use
 // One column problem per lane.  Word i of a lane's shared memory is at
 // 32 i + lane, so that any index of any lane hits its own bank.
-template <int MAXI_, int MAXJ_>
+template <int MAXI_, int MAXJ_, bool ADJ = false>
 struct SimtShape {
     static constexpr int MAXI = MAXI_, MAXJ = MAXJ_;
     static constexpr int ROWS = MAXI + 1;                // and the row of the padding entries
-    static constexpr int LW = (tri(MAXJ + 1) + 3) & ~3;  // rows 0..MAXJ of [G b], then of L
+    // rows 0..MAXJ of [G b], then of L (the adjoint's r takes their place at the end)
+    static constexpr int LMIN = ADJ && 2 * ROWS > tri(MAXJ + 1) ? 2 * ROWS : tri(MAXJ + 1);
+    static constexpr int LW = (LMIN + 3) & ~3;
     static constexpr int RW = LW;                        // r in FP64 (2 words a row); w2 during the Gram pass
     static constexpr int W4 = (LW - 2 * ROWS) & ~3;      // w4 (4 words a row: the end of L, and r) during the Gram pass
     static constexpr int TAB = LW + 2 * ROWS;            // columns of J
-    static constexpr int WORDS = TAB + MAXJ;
-    static_assert(MAXJ % 2 == 1 && RW % 2 == 0, "shape");
+    static constexpr int XD = (TAB + MAXJ + 1) & ~1;     // the adjoint's FP64 vectors over J
+    static constexpr int WORDS = ADJ ? XD + 4 * MAXJ : TAB + MAXJ;
+    static_assert(MAXJ % 2 == 1 && RW % 2 == 0 && XD % 2 == 0, "shape");
     // the row groups of four that leave w4 alone
     static constexpr int Q4 = [] {
         int q = 0;
@@ -73,168 +75,170 @@ struct Ent {
     int i[W];
 };
 
+// One column problem: its data and the steps shared by the build and its adjoint.
 template <class SH, int W>
-__global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, int bin) {
-    constexpr int MAXI = SH::MAXI, MAXJ = SH::MAXJ;
-    extern __shared__ __align__(16) float smem_f[];
-    const int lane = threadIdx.x;
-    float *S = smem_f + lane;  // word i of this lane: S[32 i]
-    double *R = reinterpret_cast<double *>(smem_f + 32 * SH::RW) + lane;
+struct Simt {
+    static constexpr int MAXI = SH::MAXI, MAXJ = SH::MAXJ;
+    const LsqArgs &args;
+    float *smem, *S;  // word i of this lane: S[32 i]
+    int lane, jj, js, n, nI, nmax, imax, zb, ze, zro, jb, roff, status;
+    int64_t poff, eoff;
+    const uint8_t *lrow;
+    float dmax, dmin;
+    bool brk;
 
-    const int w0 = args.bin_off[bin] + (args.item_hi > 0 ? args.item_lo : 0);
-    const int total = args.item_hi > 0 ? args.item_hi - args.item_lo : args.bin_off[bin + 1] - w0;
-    const int32_t *work = args.work + w0;
-    for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
-        const bool valid = base + lane < total;
-        const int jj = work[valid ? base + lane : base];  // (idle lanes repeat a column and write nothing)
+    __device__ __forceinline__ Simt(const LsqArgs &a, float *sm, int ln) : args(a), smem(sm), S(sm + ln), lane(ln) {}
+
+    __device__ __forceinline__ void begin(int col) {
+        jj = col;
         const int kmap = jj / args.n;
         const int jl = jj - kmap * args.n;
-        const int js = args.shadow_shared ? jl : jj;
-        const int64_t poff = args.shadow_shared ? (int64_t)kmap * args.map_nnz_pat : 0;
-        const int64_t eoff = args.shadow_shared ? (int64_t)kmap * args.ell_map : 0;
-        const int roff = kmap * args.n;
+        js = args.shadow_shared ? jl : jj;
+        poff = args.shadow_shared ? (int64_t)kmap * args.map_nnz_pat : 0;
+        eoff = args.shadow_shared ? (int64_t)kmap * args.ell_map : 0;
+        roff = kmap * args.n;
         const int zc = args.zbig ? jj : jl;
-        const int jb = args.jcp[js], n = args.jcp[js + 1] - jb, nI = args.icnt[js];
-        const int zb = args.zcp[zc], ze = args.zcp[zc + 1];
-        const int nmax = __reduce_max_sync(0xffffffffu, n);
-        const int imax = __reduce_max_sync(0xffffffffu, nI);
-        int status = kStOk;
+        zro = (args.shadow_shared ? 0 : roff) - (args.zbig ? roff : 0);
+        jb = args.jcp[js];
+        n = args.jcp[js + 1] - jb;
+        nI = args.icnt[js];
+        zb = args.zcp[zc];
+        ze = args.zcp[zc + 1];
+        nmax = __reduce_max_sync(0xffffffffu, n);
+        imax = __reduce_max_sync(0xffffffffu, nI);
+        status = kStOk;
         // the columns of J (past them the first one again: its values meet
         // padding rows there)
         for (int c = 0; c < nmax; ++c) S[32 * (SH::TAB + c)] = __int_as_float(args.jri[jb + (c < n ? c : 0)]);
-        const uint8_t *lrow = args.lrow_t + ((int64_t)(js >> 5) * kLTile) * 32 + (js & 31);
-        auto ell = [&](int c) -> int64_t {
-            const int col = __float_as_int(S[32 * (SH::TAB + c)]);
-            return eoff + (int64_t)(col >> 5) * (32 * W) + (col & 31);
-        };
-        auto fetch32 = [&](Ent<float, W> &e, int c) {
-            const float *v = args.kev32 + ell(c);
-            const uint8_t *l = lrow + c * (32 * W);
+        lrow = args.lrow_t + ((int64_t)(js >> 5) * kLTile) * 32 + (js & 31);
+    }
+    __device__ __forceinline__ int64_t ell(int c) const {
+        const int col = __float_as_int(S[32 * (SH::TAB + c)]);
+        return eoff + (int64_t)(col >> 5) * (32 * W) + (col & 31);
+    }
+    template <typename T>
+    __device__ __forceinline__ void fetch(Ent<T, W> &e, int c) const {
+        const T *v;
+        if constexpr (sizeof(T) == 4) v = args.kev32 + ell(c);
+        else v = args.kev + ell(c);
+        const uint8_t *l = lrow + c * (32 * W);
 #pragma unroll
-            for (int u = 0; u < W; ++u) e.v[u] = v[32 * u];
+        for (int u = 0; u < W; ++u) e.v[u] = v[32 * u];
 #pragma unroll
-            for (int u = 0; u < W; ++u) e.i[u] = l[32 * u];
-        };
-        auto fetch64 = [&](Ent<double, W> &e, int c) {
-            const double *v = args.kev + ell(c);
-            const uint8_t *l = lrow + c * (32 * W);
-#pragma unroll
-            for (int u = 0; u < W; ++u) e.v[u] = v[32 * u];
-#pragma unroll
-            for (int u = 0; u < W; ++u) e.i[u] = l[32 * u];
-        };
-        const int zro = (args.shadow_shared ? 0 : roff) - (args.zbig ? roff : 0);
-        auto target_row = [&](int t) -> int {
-            int i;
-            if (args.zloc && t - zb < kZCap) {
-                i = args.zloc[(int64_t)js * kZCap + (t - zb)];
-                if (i == kZOutside) return -1;
-                if (i >= nI) {  // impossible for a consistent shadow: never index out of bounds
-                    status = kStUnsupported;
-                    return -1;
-                }
-                return i;
+        for (int u = 0; u < W; ++u) e.i[u] = l[32 * u];
+    }
+    // f(entries, c) for the columns c < end, the next one's entries loaded
+    // while this one's are used
+    template <typename T, class F>
+    __device__ __forceinline__ void columns(int end, F &&f) const {
+        Ent<T, W> E[2];
+        fetch(E[0], 0);
+        for (int c = 0; c < end; c += 2) {
+            if (c + 1 < end) fetch(E[1], c + 1);
+            f(E[0], c);
+            if (c + 1 < end) {
+                if (c + 2 < end) fetch(E[0], c + 2);
+                f(E[1], c + 1);
             }
-            return find_sorted(args.ish + (int64_t)js * kICap, nI, args.zri[t] + zro);
-        };
-        // ---- [G b] = [B c]^T B in FP32: NW columns q of [B c] at a time
-        // dense in w, their products with every column c <= q
-        auto gram = [&](auto nw_, int qbeg, int qend, float *w) {
-            constexpr int NW = decltype(nw_)::value;
-            for (int i = 0; i < imax; ++i)
+        }
+    }
+    __device__ __forceinline__ int target_row(int t) {
+        if (args.zloc && t - zb < kZCap) {
+            const int i = args.zloc[(int64_t)js * kZCap + (t - zb)];
+            if (i == kZOutside) return -1;
+            if (i >= nI) {  // impossible for a consistent shadow: never index out of bounds
+                status = kStUnsupported;
+                return -1;
+            }
+            return i;
+        }
+        return find_sorted(args.ish + (int64_t)js * kICap, nI, args.zri[t] + zro);
+    }
+
+    // [G b] = [B c]^T B in FP32: NW columns q of [B c] at a time dense in w,
+    // their products with every column c <= q (RHS: with c as column n)
+    template <int NW, bool RHS>
+    __device__ __forceinline__ void gram(int qbeg, int qend, float *w) {
+        for (int i = 0; i < imax; ++i)
 #pragma unroll
-                for (int t = 0; t < NW; ++t) w[32 * NW * i + t] = 0.f;
+            for (int t = 0; t < NW; ++t) w[32 * NW * i + t] = 0.f;
 #pragma unroll
-            for (int t = 0; t < NW; ++t) w[32 * NW * MAXI + t] = 0.f;
-            for (int q0 = qbeg; q0 < qend; q0 += NW) {
-                if (q0 > nmax) break;
-                const int cend = min(q0 + NW, nmax);
-                Ent<float, W> E[kAhead + 1];
-                fetch32(E[0], 0);
-                                int rows[NW][W];
+        for (int t = 0; t < NW; ++t) w[32 * NW * MAXI + t] = 0.f;
+        for (int q0 = qbeg; q0 < qend; q0 += NW) {
+            if (q0 >= nmax + (RHS ? 1 : 0)) break;
+            const int cend = min(q0 + NW, nmax);
+            int rows[NW][W];
 #pragma unroll
-                for (int t = 0; t < NW; ++t) {
-                    const int q = q0 + t;
-                    if (q < nmax) {
-                        Ent<float, W> e;
-                        fetch32(e, q);
-#pragma unroll
-                        for (int u = 0; u < W; ++u) {
-                            rows[t][u] = e.i[u];
-                            if (q < n) w[32 * NW * e.i[u] + t] = e.v[u];
-                        }
-                    }
-                    w[32 * NW * MAXI + t] = 0.f;  // (padding entries wrote there)
-                    if (q == n)
-                        for (int z = zb; z < ze; ++z) {
-                            const int i = target_row(z);
-                            if (i >= 0) w[32 * NW * i + t] = args.zcv32[z];
-                        }
-                }
-                auto dots = [&](const Ent<float, W> &e, int c) {
-                    float acc[NW] = {};
+            for (int t = 0; t < NW; ++t) {
+                const int q = q0 + t;
+                if (q < nmax) {
+                    Ent<float, W> e;
+                    fetch(e, q);
 #pragma unroll
                     for (int u = 0; u < W; ++u) {
-                        const float *wr = w + 32 * NW * e.i[u];
-                        if constexpr (NW == 4) {
-                            const float4 x = *reinterpret_cast<const float4 *>(wr);
-                            acc[0] = fmaf(e.v[u], x.x, acc[0]);
-                            acc[1] = fmaf(e.v[u], x.y, acc[1]);
-                            acc[2] = fmaf(e.v[u], x.z, acc[2]);
-                            acc[3] = fmaf(e.v[u], x.w, acc[3]);
-                        } else {
-                            const float2 x = *reinterpret_cast<const float2 *>(wr);
-                            acc[0] = fmaf(e.v[u], x.x, acc[0]);
-                            acc[1] = fmaf(e.v[u], x.y, acc[1]);
-                        }
-                    }
-                    const int b = tri(q0) + c;
-#pragma unroll
-                    for (int t = 0; t < NW; ++t)
-                        if (q0 + t >= c && q0 + t <= MAXJ) S[32 * (b + t * q0 + tri(t))] = acc[t];
-                };
-                for (int c = 0; c < cend; c += kAhead + 1) {
-#pragma unroll
-                    for (int k = 0; k < kAhead + 1; ++k) {
-                        if (c + k < cend) {
-                            if (c + k + kAhead < cend) fetch32(E[(k + kAhead) % (kAhead + 1)], c + k + kAhead);
-                            dots(E[k], c + k);
-                        }
+                        rows[t][u] = e.i[u];
+                        if (q < n) w[32 * NW * e.i[u] + t] = e.v[u];
                     }
                 }
-                // clear the block's columns of w
-#pragma unroll
-                for (int t = 0; t < NW; ++t) {
-                    const int q = q0 + t;
-                    if (q < nmax) {
-#pragma unroll
-                        for (int u = 0; u < W; ++u) w[32 * NW * rows[t][u] + t] = 0.f;
+                w[32 * NW * MAXI + t] = 0.f;  // (padding entries wrote there)
+                if (RHS && q == n)
+                    for (int z = zb; z < ze; ++z) {
+                        const int i = target_row(z);
+                        if (i >= 0) w[32 * NW * i + t] = args.zcv32[z];
                     }
-                    if (q == n)
-                        for (int z = zb; z < ze; ++z) {
-                            const int i = target_row(z);
-                            if (i >= 0) w[32 * NW * i + t] = 0.f;
-                        }
-                }
             }
-        };
-        gram(std::integral_constant<int, 4>{}, 0, SH::Q4, smem_f + 32 * SH::W4 + 4 * lane);
-        gram(std::integral_constant<int, 2>{}, SH::Q4, MAXJ + 1, smem_f + 32 * SH::RW + 2 * lane);
-        // ---- r = c in FP64
-        double out2 = 0.0;
-        for (int i = 0; i < imax; ++i) R[32 * i] = 0.0;
-        R[32 * MAXI] = 0.0;
-        for (int z = zb; z < ze; ++z) {
-            const int i = target_row(z);
-            const double v = args.zcv[z];
-            if (i >= 0) R[32 * i] = v;
-            else out2 = fma(v, v, out2);
+            columns<float>(cend, [&](const Ent<float, W> &e, int c) {
+                float acc[NW] = {};
+#pragma unroll
+                for (int u = 0; u < W; ++u) {
+                    const float *wr = w + 32 * NW * e.i[u];
+                    if constexpr (NW == 4) {
+                        const float4 x = *reinterpret_cast<const float4 *>(wr);
+                        acc[0] = fmaf(e.v[u], x.x, acc[0]);
+                        acc[1] = fmaf(e.v[u], x.y, acc[1]);
+                        acc[2] = fmaf(e.v[u], x.z, acc[2]);
+                        acc[3] = fmaf(e.v[u], x.w, acc[3]);
+                    } else {
+                        const float2 x = *reinterpret_cast<const float2 *>(wr);
+                        acc[0] = fmaf(e.v[u], x.x, acc[0]);
+                        acc[1] = fmaf(e.v[u], x.y, acc[1]);
+                    }
+                }
+                const int b = tri(q0) + c;
+#pragma unroll
+                for (int t = 0; t < NW; ++t)
+                    if (q0 + t >= c && q0 + t <= MAXJ) S[32 * (b + t * q0 + tri(t))] = acc[t];
+            });
+            // clear the block's columns of w
+#pragma unroll
+            for (int t = 0; t < NW; ++t) {
+                const int q = q0 + t;
+                if (q < nmax) {
+#pragma unroll
+                    for (int u = 0; u < W; ++u) w[32 * NW * rows[t][u] + t] = 0.f;
+                }
+                if (RHS && q == n)
+                    for (int z = zb; z < ze; ++z) {
+                        const int i = target_row(z);
+                        if (i >= 0) w[32 * NW * i + t] = 0.f;
+                    }
+            }
         }
-        // ---- G = L L^T, two rows at a time in registers; the row of b gives
-        // y = L^{-1} b.  The diagonal holds 1 / L_kk
-        float dmax = 0.f, dmin = FLT_MAX;
-        bool brk = false;
-        for (int q0 = 0; q0 <= nmax; q0 += 2) {
+    }
+    template <bool RHS>
+    __device__ __forceinline__ void gram_all() {
+        gram<4, RHS>(0, SH::Q4, smem + 32 * SH::W4 + 4 * lane);
+        gram<2, RHS>(SH::Q4, MAXJ + 1, smem + 32 * SH::RW + 2 * lane);
+    }
+
+    // G = L L^T, two rows at a time in registers (RHS: the row of b gives
+    // y = L^{-1} b).  The diagonal holds 1 / L_kk
+    template <bool RHS>
+    __device__ __forceinline__ void factor() {
+        dmax = 0.f;
+        dmin = FLT_MAX;
+        brk = false;
+        for (int q0 = 0; q0 < nmax + (RHS ? 1 : 0); q0 += 2) {
             const int b0 = tri(q0), b1 = tri(q0 + 1);
             float a0[MAXJ], a1[MAXJ];
             float t00 = S[32 * (b0 + q0)], t10 = S[32 * (b1 + q0)], t11 = S[32 * (b1 + q0 + 1)];
@@ -263,15 +267,6 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
                 t10 = fmaf(-a0[j], a1[j], t10);
                 t11 = fmaf(-a1[j], a1[j], t11);
             }
-            auto pivot = [&](int q, float t) -> float {
-                if (q >= n) return 0.f;
-                // (past a breakdown every pivot is NaN: the FP64 re-solve decides)
-                if (!brk && !(fabsf(t) <= FLT_MAX)) status = max(status, (int)kStNonfinite);
-                brk = brk || !(t > 0.f);
-                dmax = fmaxf(dmax, t);
-                dmin = fminf(dmin, t);
-                return rsqrtf(t);
-            };
             const float i0 = pivot(q0, t00);
             const float l10 = t10 * i0;
             const float i1 = pivot(q0 + 1, fmaf(-l10, l10, t11));
@@ -279,46 +274,133 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
             S[32 * (b1 + q0)] = l10;
             S[32 * (b1 + q0 + 1)] = i1;
         }
-        const float kap2 = dmax / dmin;  // a lower bound on kappa(B)^2
-        const int xb = tri(n);           // y, then each product's x and g, in the row of b
+    }
+    __device__ __forceinline__ float pivot(int q, float t) {
+        if (q >= n) return 0.f;
+        // (past a breakdown every pivot is NaN: the re-solve decides)
+        if (!brk && !(fabsf(t) <= FLT_MAX)) status = max(status, (int)kStNonfinite);
+        brk = brk || !(t > 0.f);
+        dmax = fmaxf(dmax, t);
+        dmin = fminf(dmin, t);
+        return rsqrtf(t);
+    }
+
+    // the vector of a product or a solve, in the row of b
+    __device__ __forceinline__ void load_x(float (&x)[MAXJ]) const {
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j) x[j] = (j < n) ? S[32 * (tri(n) + j)] : 0.f;
+    }
+    __device__ __forceinline__ void store_x(const float (&x)[MAXJ]) {
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j)
+            if (j < n) S[32 * (tri(n) + j)] = x[j];
+    }
+    __device__ __forceinline__ void back(float (&x)[MAXJ]) const {  // L^T x = y
+#pragma unroll
+        for (int j = MAXJ - 1; j >= 0; --j) {
+            if (j >= nmax) continue;
+            if (j < n) {
+                const float xj = x[j] * S[32 * (tri(j) + j)];
+                x[j] = xj;
+#pragma unroll
+                for (int k = 0; k < j; ++k) x[k] = fmaf(-S[32 * (tri(j) + k)], xj, x[k]);
+            }
+        }
+    }
+    __device__ __forceinline__ void fwd(float (&x)[MAXJ]) const {  // L y = g
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j) {
+            if (j >= nmax) break;
+            float s = x[j], p = 0.f;
+#pragma unroll
+            for (int k = 0; k < j; ++k) {
+                const float l = S[32 * (tri(j) + k)];
+                if (k & 1) p = fmaf(-l, x[k], p);
+                else s = fmaf(-l, x[k], s);
+            }
+            x[j] = (j < n) ? (s + p) * S[32 * (tri(j) + j)] : 0.f;
+        }
+    }
+
+    // r += B x (FP64), column by column; x(c): the factor of column c (0 past n)
+    template <class X>
+    __device__ __forceinline__ void add_bx(double *R, X &&x) const {
+        columns<double>(nmax, [&](const Ent<double, W> &e, int c) {
+            const double xc = x(c);
+            double rv[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) rv[u] = R[32 * e.i[u]];
+#pragma unroll
+            for (int u = 0; u < W; ++u) rv[u] = fma(e.v[u], xc, rv[u]);
+#pragma unroll
+            for (int u = 0; u < W; ++u) R[32 * e.i[u]] = rv[u];
+        });
+    }
+    // put(c, (B^T r)_c) (FP64)
+    template <class F>
+    __device__ __forceinline__ void bt_r(const double *R, F &&put) const {
+        columns<double>(nmax, [&](const Ent<double, W> &e, int c) {
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                const double rr = R[32 * e.i[u]];
+                if (u % 3 == 0) s0 = fma(e.v[u], rr, s0);
+                else if (u % 3 == 1) s1 = fma(e.v[u], rr, s1);
+                else s2 = fma(e.v[u], rr, s2);
+            }
+            if (c < n) put(c, s0 + s1 + s2);
+        });
+    }
+    // r = c in FP64; returns the target's entries outside the shadow, squared
+    __device__ __forceinline__ double target(double *R) {
+        double out2 = 0.0;
+        for (int i = 0; i < imax; ++i) R[32 * i] = 0.0;
+        R[32 * MAXI] = 0.0;
+        for (int z = zb; z < ze; ++z) {
+            const int i = target_row(z);
+            const double v = args.zcv[z];
+            if (i >= 0) R[32 * i] = v;
+            else out2 = fma(v, v, out2);
+        }
+        return out2;
+    }
+};
+
+template <class SH, int W>
+__global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, int bin) {
+    constexpr int MAXJ = SH::MAXJ;
+    extern __shared__ __align__(16) float smem_f[];
+    const int lane = threadIdx.x;
+    double *R = reinterpret_cast<double *>(smem_f + 32 * SH::RW) + lane;
+    Simt<SH, W> C(args, smem_f, lane);
+    float *S = C.S;
+
+    const int w0 = args.bin_off[bin] + (args.item_hi > 0 ? args.item_lo : 0);
+    const int total = args.item_hi > 0 ? args.item_hi - args.item_lo : args.bin_off[bin + 1] - w0;
+    const int32_t *work = args.work + w0;
+    for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
+        const bool valid = base + lane < total;
+        C.begin(work[valid ? base + lane : base]);  // (idle lanes repeat a column and write nothing)
+        const int n = C.n;
+        C.template gram_all<true>();
+        const double out2 = C.target(R);
+        C.template factor<true>();
+        const bool brk = C.brk;
+        const float kap2 = C.dmax / C.dmin;  // a lower bound on kappa(B)^2
+        // factor tape: R = L^T, packed (its rows are L's columns), also past a
+        // zero or non-finite pivot
+        if (args.fac_mode == kTapeRecord && valid) {
+            float *dst = reinterpret_cast<float *>(args.fac) + args.fac_off[C.jj];
+            for (int k = 0; k < n; ++k) {
+                const float inv = S[32 * (tri(k) + k)];
+                *dst++ = inv == 0.f ? inv : 1.f / inv;
+                for (int c = k + 1; c < n; ++c) *dst++ = S[32 * (tri(c) + k)];
+            }
+        }
+        const int xb = tri(n);
         float x[MAXJ];
-        auto load_x = [&]() {
-#pragma unroll
-            for (int j = 0; j < MAXJ; ++j) x[j] = (j < n) ? S[32 * (xb + j)] : 0.f;
-        };
-        auto store_x = [&]() {
-#pragma unroll
-            for (int j = 0; j < MAXJ; ++j)
-                if (j < n) S[32 * (xb + j)] = x[j];
-        };
-        auto back = [&]() {  // L^T x = y
-#pragma unroll
-            for (int j = MAXJ - 1; j >= 0; --j) {
-                if (j >= nmax) continue;
-                if (j < n) {
-                    const float xj = x[j] * S[32 * (tri(j) + j)];
-                    x[j] = xj;
-#pragma unroll
-                    for (int k = 0; k < j; ++k) x[k] = fmaf(-S[32 * (tri(j) + k)], xj, x[k]);
-                }
-            }
-        };
-        auto fwd = [&]() {  // L y = g
-#pragma unroll
-            for (int j = 0; j < MAXJ; ++j) {
-                if (j >= nmax) break;
-                float s = x[j], p = 0.f;
-#pragma unroll
-                for (int k = 0; k < j; ++k) {
-                    const float l = S[32 * (tri(j) + k)];
-                    if (k & 1) p = fmaf(-l, x[k], p);
-                    else s = fmaf(-l, x[k], s);
-                }
-                x[j] = (j < n) ? (s + p) * S[32 * (tri(j) + j)] : 0.f;
-            }
-        };
-        load_x();
-        back();
+        C.load_x(x);
+        C.back(x);
         double m[MAXJ];
         float msq = 0.f;
 #pragma unroll
@@ -332,48 +414,13 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
         const int steps = autoref ? 1 : args.refine_steps;
         float da2 = 0.f, dprev2 = 0.f;
         for (int step = 0; step <= steps; ++step) {
-            store_x();
-            Ent<double, W> E[kAhead + 1];
-            // r -= B x (FP64), column by column
-            fetch64(E[0], 0);
-            for (int c = 0; c < nmax; c += kAhead + 1) {
-#pragma unroll
-                for (int k = 0; k < kAhead + 1; ++k) {
-                    if (c + k < nmax) {
-                        if (c + k + kAhead < nmax) fetch64(E[(k + kAhead) % (kAhead + 1)], c + k + kAhead);
-                        const double xc = c + k < n ? -widen(S[32 * (xb + c + k)]) : 0.0;
-                        double rv[W];
-#pragma unroll
-                        for (int u = 0; u < W; ++u) rv[u] = R[32 * E[k].i[u]];
-#pragma unroll
-                        for (int u = 0; u < W; ++u) rv[u] = fma(E[k].v[u], xc, rv[u]);
-#pragma unroll
-                        for (int u = 0; u < W; ++u) R[32 * E[k].i[u]] = rv[u];
-                    }
-                }
-            }
-            // g = B^T r (FP64, rounded to FP32)
-            fetch64(E[0], 0);
-            for (int c = 0; c < nmax; c += kAhead + 1) {
-#pragma unroll
-                for (int k = 0; k < kAhead + 1; ++k) {
-                    if (c + k < nmax) {
-                        if (c + k + kAhead < nmax) fetch64(E[(k + kAhead) % (kAhead + 1)], c + k + kAhead);
-                        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-#pragma unroll
-                        for (int u = 0; u < W; ++u) {
-                            const double rr = R[32 * E[k].i[u]];
-                            if (u % 3 == 0) s0 = fma(E[k].v[u], rr, s0);
-                            else if (u % 3 == 1) s1 = fma(E[k].v[u], rr, s1);
-                            else s2 = fma(E[k].v[u], rr, s2);
-                        }
-                        if (c + k < n) S[32 * (xb + c + k)] = narrow_trunc(s0 + s1 + s2);
-                    }
-                }
-            }
-            load_x();
-            fwd();
-            back();
+            // r -= B x, g = B^T r (rounded to FP32), d = (L L^T)^{-1} g, m += d
+            C.store_x(x);
+            C.add_bx(R, [&](int c) { return c < n ? -widen(S[32 * (xb + c)]) : 0.0; });
+            C.bt_r(R, [&](int c, double g) { S[32 * (xb + c)] = narrow_trunc(g); });
+            C.load_x(x);
+            C.fwd(x);
+            C.back(x);
             float dsq = 0.f;
 #pragma unroll
             for (int j = 0; j < MAXJ; ++j) {
@@ -402,16 +449,17 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
 #pragma unroll
                 for (int j = 0; j < MAXJ; ++j)
                     if (j < n) dg = fmaf(x[j], S[32 * (xb + j)], dg);
-                for (int i = 0; i < nI; ++i) r2 = fma(R[32 * i], R[32 * i], r2);
+                for (int i = 0; i < C.nI; ++i) r2 = fma(R[32 * i], R[32 * i], r2);
                 r2 -= widen(dg);
             }
             dprev2 = dsq;
         }
         if (autoref && brk) redo = true;
         // ---- outputs
+        int status = C.status;
         if (valid) {
             if (args.refine_used)
-                args.refine_used[jj] = (uint8_t)((fallback && status == kStOk) ? kAutoSteps + 1 : (steps < 2 ? steps : 2));
+                args.refine_used[C.jj] = (uint8_t)((fallback && status == kStOk) ? kAutoSteps + 1 : (steps < 2 ? steps : 2));
             bool nf = !finite64(r2);
 #pragma unroll
             for (int j = 0; j < MAXJ; ++j) nf = nf || (j < n && !finite64(m[j]));
@@ -420,10 +468,126 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
             if (status == kStOk && redo) status = kStStep2;
 #pragma unroll
             for (int j = 0; j < MAXJ; ++j)
-                if (j < n) args.mval[args.csr_pos[jb + j] + poff] = (status == kStOk) ? m[j] : 0.0;
-            args.colres[jj] = (status == kStOk) ? (r2 > 0.0 ? r2 : 0.0) + out2 : 0.0;
-            args.colstat[jj] = status;
+                if (j < n) args.mval[args.csr_pos[C.jb + j] + C.poff] = (status == kStOk) ? m[j] : 0.0;
+            args.colres[C.jj] = (status == kStOk) ? (r2 > 0.0 ? r2 : 0.0) + out2 : 0.0;
+            args.colstat[C.jj] = status;
         }
+    }
+}
+
+// The adjoint of the columns (adjoint_core.cuh says what it computes): lambda
+// from the Cholesky factor with FP64 corrections, w = B lambda and r = c - B m
+// in FP64, dL/dB in gather order.  The Cholesky factor contracts an error by
+// rho, about u_32 kappa^2 per correction; a column whose estimate of rho is above
+// kAdjRho (level-1 columns: 1e-6) goes to rest, for the QR kernel.
+constexpr float kAdjRho = 1e-5f;
+
+template <class SH, int W>
+__global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs args, int bin, int32_t *rest,
+                                                                    int32_t *rest_off) {
+    constexpr int MAXI = SH::MAXI, MAXJ = SH::MAXJ;
+    extern __shared__ __align__(16) float smem_f[];
+    const int lane = threadIdx.x;
+    double *Wv = reinterpret_cast<double *>(smem_f + 32 * SH::RW) + lane;  // B lambda
+    double *R = reinterpret_cast<double *>(smem_f) + lane;                 // r, once L is done with
+    double *X = reinterpret_cast<double *>(smem_f + 32 * SH::XD) + lane;   // m, then lambda's column factors
+    static_assert(2 * SH::ROWS <= SH::LW, "r takes L's place");
+    Simt<SH, W> C(args, smem_f, lane);
+    float *S = C.S;
+    const int w0 = args.bin_off[bin], total = args.bin_off[bin + 1] - w0;
+    const int32_t *work = args.work + w0;
+    const double rho = args.resid_weight;
+    for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
+        const bool valid = base + lane < total;
+        C.begin(work[valid ? base + lane : base]);  // (idle lanes repeat a column and write nothing)
+        const int n = C.n;
+        C.template gram_all<false>();
+        C.template factor<false>();
+        const float kap2 = C.dmax / C.dmin;
+        const int xb = tri(n);
+        // ---- lambda = G^{-1} g: w = B lambda grows with it
+        double gq[MAXJ], lq[MAXJ];
+        float x[MAXJ];
+        float l2 = 0.f, d2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j) {
+            gq[j] = (j < n && args.dmval) ? args.dmval[args.csr_pos[C.jb + j] + C.poff] : 0.0;
+            x[j] = narrow_trunc(gq[j]);
+        }
+        for (int i = 0; i < C.imax; ++i) Wv[32 * i] = 0.0;
+        Wv[32 * MAXI] = 0.0;
+        C.fwd(x);
+        C.back(x);
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j) {
+            lq[j] = widen(x[j]);
+            l2 = fmaf(x[j], x[j], l2);
+        }
+        const int corr = args.refine_steps < 2 ? args.refine_steps + 1 : args.refine_steps;
+        for (int step = 0; step <= corr; ++step) {
+            C.store_x(x);
+            C.add_bx(Wv, [&](int c) { return c < n ? widen(S[32 * (xb + c)]) : 0.0; });
+            if (step == corr) break;
+            // correction: lambda += (L L^T)^{-1} (g - B^T w)
+            C.bt_r(Wv, [&](int c, double t) { X[32 * c] = t; });
+#pragma unroll
+            for (int j = 0; j < MAXJ; ++j) x[j] = j < n ? narrow_trunc(gq[j] - X[32 * j]) : 0.f;
+            C.fwd(x);
+            C.back(x);
+            float s = 0.f;
+#pragma unroll
+            for (int j = 0; j < MAXJ; ++j) {
+                lq[j] += widen(x[j]);
+                s = fmaf(x[j], x[j], s);
+            }
+            if (step == 0) d2 = s;
+        }
+        // ---- does the QR kernel have to take the column?
+        const float rk = (float)(kRhoSafety * kU32) * kap2;
+        bool leave = C.status == kStOk && (C.brk || !(rk <= kAdjRho) || !(16.f * d2 <= kAdjRho * kAdjRho * l2));
+        if (valid && leave) rest[atomicAdd(&rest_off[1], 1)] = C.jj;
+        // ---- r = c - B m
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j)
+            if (j < n) X[32 * j] = args.mval[args.csr_pos[C.jb + j] + C.poff];
+        C.target(R);
+        C.add_bx(R, [&](int c) { return c < n ? -X[32 * c] : 0.0; });
+        const bool write = valid && !leave && C.status == kStOk;
+        // ---- dL/dB(i, c) = r_i (lambda_c - 2 rho m_c) - w_i m_c, and where each column's block starts
+        const int64_t blk = args.dB_off[C.jj];
+#pragma unroll
+        for (int j = 0; j < MAXJ; ++j)  // (x: lambda in FP64 words is not kept: the factor goes with m)
+            if (j < n) X[32 * (MAXJ + j)] = fma(-2.0 * rho, X[32 * j], lq[j]);
+        int e0 = 0;
+        for (int c = 0; c < C.nmax; ++c) {
+            if (c >= n) break;
+            const double ac = X[32 * (MAXJ + c)], nm = -X[32 * c];
+            const uint8_t *l = C.lrow + c * (32 * W);
+            int i[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) i[u] = l[32 * u];
+            int len = 0;
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                const double v = fma(R[32 * i[u]], ac, Wv[32 * i[u]] * nm);
+                if (write && i[u] != MAXI) args.dB[blk + e0 + u] = v;
+                len += i[u] != MAXI ? 1 : 0;
+            }
+            if (write) args.dbase[args.csr_pos[C.jb + c] + C.poff] = blk + e0;
+            e0 += len;
+        }
+        if (args.dmres) C.bt_r(R, [&](int c, double t) {
+            if (write) args.dmres[args.csr_pos[C.jb + c] + C.poff] = -2.0 * rho * t;
+        });
+        // ---- dL/dA_0(:, j)
+        if (write) {
+            const int64_t zoff = args.zbig ? 0 : (int64_t)(C.roff / args.n) * args.znnz;
+            for (int t = C.zb; t < C.ze; ++t) {
+                const int i = C.target_row(t);
+                args.dzval[zoff + t] = (i >= 0) ? Wv[32 * i] + 2.0 * rho * R[32 * i] : 2.0 * rho * args.zcv[t];
+            }
+        }
+        if (valid && !leave) args.colstat[C.jj] = C.status;
     }
 }
 
@@ -441,6 +605,21 @@ cudaError_t launch_simt(sam_handle h, const LsqArgs &a, int bin) {
     kern<<<per_sm * handle_sms(h), 32, smem, handle_stream(h)>>>(a, bin);
     count_launch(h);
     profile_end(h, bin);
+    return cudaGetLastError();
+}
+
+template <class SH, int W>
+cudaError_t launch_adjoint(sam_handle h, const LsqArgs &a, int bin) {
+    const size_t smem = SH::BYTES;
+    auto kern = adjoint_simt_kernel<SH, W>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    kern<<<per_sm * handle_sms(h), 32, smem, handle_stream(h)>>>(a, bin, a.dense_list, a.dense_off);
+    count_launch(h);
     return cudaGetLastError();
 }
 
@@ -519,6 +698,23 @@ cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin) {
         case 7: return launch_width<7>(h, args, bin);
         case 9: return launch_width<9>(h, args, bin);
         case kEllW: return launch_width<kEllW>(h, args, bin);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// the columns left over go to dense_list, their number to dense_off[1] (from 0)
+cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args) {
+    cudaError_t e;
+    switch (args.ell_w) {
+#define SAM_ADJ_W(WW)                                                                                          \
+    case WW:                                                                                                   \
+        if ((e = launch_adjoint<SimtShape<14, 5, true>, WW>(h, args, 0)) != cudaSuccess) return e;              \
+        return launch_adjoint<SimtShape<26, 9, true>, WW>(h, args, 1);
+        SAM_ADJ_W(5)
+        SAM_ADJ_W(7)
+        SAM_ADJ_W(9)
+        SAM_ADJ_W(kEllW)
+#undef SAM_ADJ_W
         default: return cudaErrorInvalidValue;
     }
 }
