@@ -216,6 +216,45 @@ __device__ __forceinline__ int group_excl_scan(int v, int ll, int *total) {
 
 // ---------------------------------------------------------- Householder QR
 
+// scale * (sum of w[t] over the RG lanes with the same high lane bits) for
+// each t < N, on all of those lanes.  Step by step each lane keeps half of
+// the values and adds its partner's: (1 - 1/RG) N additions in place of
+// log2(RG) N, N / RG products in place of N, and the sums are those of the
+// butterfly, bit for bit.
+template <typename T, int N, int RG>
+struct RowReduce {
+    static __device__ __forceinline__ void run(T (&w)[N], int rg, T scale) {
+        constexpr int H = (N + 1) / 2;
+        T v[H];
+        const bool odd = rg & 1;
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const T hi = 2 * i + 1 < N ? w[2 * i + 1 < N ? 2 * i + 1 : 0] : w[2 * i];
+            v[i] = (odd ? hi : w[2 * i]) + shfl_xor(odd ? w[2 * i] : hi, 1);
+        }
+        const int base = (int)(threadIdx.x & 31) & ~(RG - 1);
+        if constexpr (RG == 2) {
+#pragma unroll
+            for (int i = 0; i < H; ++i) v[i] *= scale;
+#pragma unroll
+            for (int t = 0; t < N; ++t) w[t] = shfl(v[t / 2], base | (2 * (t / 2) + 1 < N ? t & 1 : 0));
+        } else {
+            static_assert(RG == 4, "row groups of two or four lanes");
+            constexpr int Q = (H + 1) / 2;
+            T x[Q];
+            const bool up = rg & 2;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const T hi = 2 * i + 1 < H ? v[2 * i + 1 < H ? 2 * i + 1 : 0] : v[2 * i];
+                x[i] = ((up ? hi : v[2 * i]) + shfl_xor(up ? v[2 * i] : hi, 2)) * scale;
+            }
+            // value t sits on lane (t & 1) + 2 ((t / 2) & 1) in x[t / 4]
+#pragma unroll
+            for (int t = 0; t < N; ++t) w[t] = shfl(x[t / 4], base | (t & 3));
+        }
+    }
+};
+
 template <class TL, int PH>
 struct QRPhase {
     using T = typename TL::T;
@@ -228,6 +267,14 @@ struct QRPhase {
     // after it (the tail) only when its row band reaches them (tiles
     // without BAND: the head is every slot, and no band is read)
     static constexpr int SE = TL::BAND && SK + (RS + 1) / 2 < RS ? SK + (RS + 1) / 2 : RS;
+
+    // FP64 tiles are bound by the FP64 pipe (a warp instruction takes an SM
+    // about 17 cycles at the measured 1.06 TFLOP/s): column k's own dot
+    // product is its norm, so its separate chain is left out, and the dot
+    // products are reduced with the fewest additions (RowReduce).  FP32 tiles
+    // are bound by latency: there the chain runs beside the dot products, and
+    // RowReduce made no difference (10-map Q1 level-2 build 5.61 / 5.66 ms).
+    static constexpr bool FP64_BOUND = sizeof(T) == 8;
 
     // band[k]: the row slot of the last row that holds an entry of columns
     // 0..k of B (Column::build_rows).  Householder reflectors 0..k leave
@@ -255,22 +302,26 @@ struct QRPhase {
                     tail = sh >= SE;
                 }
                 // squared norm of column k below the diagonal (two chains)
-                T sig0 = T(0), sig1 = T(0);
+                T sig = T(0);
+                if constexpr (!FP64_BOUND) {
+                    T sig0 = T(0), sig1 = T(0);
 #pragma unroll
-                for (int s = SK; s < SE; ++s) {
-                    T x = a[s][TK];
-                    if (s == SK) x = (rg > rk) ? x : T(0);
-                    if ((s - SK) & 1) sig1 = fma(x, x, sig1); else sig0 = fma(x, x, sig0);
-                }
-                if (tail) {
-#pragma unroll
-                    for (int s = SE; s < RS; ++s) {
-                        if ((s - SK) & 1) sig1 = fma(a[s][TK], a[s][TK], sig1); else sig0 = fma(a[s][TK], a[s][TK], sig0);
+                    for (int s = SK; s < SE; ++s) {
+                        T x = a[s][TK];
+                        if (s == SK) x = (rg > rk) ? x : T(0);
+                        if ((s - SK) & 1) sig1 = fma(x, x, sig1); else sig0 = fma(x, x, sig0);
                     }
-                }
-                T sig = sig0 + sig1;
+                    if (tail) {
 #pragma unroll
-                for (int o = 1; o < RG; o <<= 1) sig += shfl_xor(sig, o);
+                        for (int s = SE; s < RS; ++s) {
+                            if ((s - SK) & 1) sig1 = fma(a[s][TK], a[s][TK], sig1);
+                            else sig0 = fma(a[s][TK], a[s][TK], sig0);
+                        }
+                    }
+                    sig = sig0 + sig1;
+#pragma unroll
+                    for (int o = 1; o < RG; o <<= 1) sig += shfl_xor(sig, o);
+                }
                 // column k of the rows below the pivot slot, from its owners,
                 // and their part of the dot products: independent of the
                 // reflector's norm, so they overlap its reductions and square
@@ -294,6 +345,12 @@ struct QRPhase {
                         for (int t = TK; t < CS; ++t) w[t - TK] = fma(x, a[s][t], w[t - TK]);
                     }
                 }
+                if constexpr (FP64_BOUND) {
+                    const T x = (rg > rk) ? a[SK][TK] : T(0);
+                    sig = fma(x, x, w[0]);
+#pragma unroll
+                    for (int o = 1; o < RG; o <<= 1) sig += shfl_xor(sig, o);
+                }
                 const T alpha = shfl(a[SK][TK], gbase + ck * RG + rk);
                 const T sigma = shfl(sig, gbase + ck * RG);
                 // reflector H = I - taup u u^T, u = x with u_k = alpha - beta
@@ -308,17 +365,23 @@ struct QRPhase {
 #pragma unroll
                     for (int t = TK; t < CS; ++t) w[t - TK] = fma(x, a[SK][t], w[t - TK]);
                 }
-                // reductions interleaved (independent shuffles in flight
-                // together), then the updates
+                if constexpr (FP64_BOUND) {
+                    // reduced over the column's RG lanes by halving the values
+                    // with the lanes (the same sums), scaled by one lane each
+                    // and handed back
+                    RowReduce<T, CS - TK, RG>::run(w, rg, taup);
+                } else {
+                    // reductions interleaved (independent shuffles in flight
+                    // together), then the updates
 #pragma unroll
-                for (int o = 1; o < RG; o <<= 1)
+                    for (int o = 1; o < RG; o <<= 1)
 #pragma unroll
-                    for (int t = TK; t < CS; ++t) w[t - TK] += shfl_xor(w[t - TK], o);
+                        for (int t = TK; t < CS; ++t) w[t - TK] += shfl_xor(w[t - TK], o);
 #pragma unroll
-                for (int t = TK; t < CS; ++t) {
-                    // columns of slots after TK are all > k (L divides CG)
-                    w[t - TK] = (t > TK || t * CG + cg > k) ? taup * w[t - TK] : T(0);
+                    for (int t = TK; t < CS; ++t) w[t - TK] *= taup;
                 }
+                // columns of slots after TK are all > k (L divides CG)
+                if (TK * CG + cg <= k) w[0] = T(0);
 #pragma unroll
                 for (int s = SK; s < SE; ++s)
 #pragma unroll
@@ -445,11 +508,20 @@ using F1 = Tile<2, 2, 13, 5, float, 26>;
 using F2 = Tile<4, 4, 10, 6, float, 40, false, true>;
 using F3 = Tile<4, 4, 13, 7, float, 52, false, true>;
 using F4 = Tile<4, 4, 16, 7, float, 64>;
-// FP64 tiles
+// FP64 tiles.  A slot costs the FP64 pipe the same whether its lanes hold
+// entries or padding, and the norm, square root and division of a reflector
+// cost it the same for one column problem per warp as for two: two problems of
+// 16 lanes (class 1: eight of 4 lanes, not four of 8) take 109 column slots for 25
+// unknowns where one of 32 took 73 each, and half the reflector overhead, at
+// 255 registers and 8 warps per SM, which still fill the pipe.  With the QR's
+// shorter sums (QRPhase) two 256^2 Q1 level-2 maps went from 16.6 to 9.46 ms,
+// eight level-1 ones from 7.30 to 4.60, a level-2 map with its residual and adjoint
+// from 27.8 to 16.2.  Class 4 (16 x 7 slots: 224 registers) keeps 32 lanes,
+// with 255 registers instead of 168 and 476 bytes of spills.
 using D0 = Tile<2, 2, 7, 3, double, 14>;
-using D1 = Tile<2, 4, 13, 3, double, 26>;
-using D2 = Tile<4, 8, 10, 3, double, 40, false, true>;
-using D3 = Tile<4, 8, 13, 4, double, 52, false, true>;
+using D1 = Tile<2, 2, 13, 5, double, 26>;
+using D2 = Tile<4, 4, 10, 6, double, 40, false, true>;
+using D3 = Tile<4, 4, 13, 7, double, 52, false, true>;
 using D4 = Tile<4, 8, 16, 4, double, 64>;
 
 // alternative shapes for the autotuner: one problem per 8 or 32 lanes
@@ -462,8 +534,8 @@ using F4b = Tile<4, 8, 16, 4, float, 64>;
 using F2L = Tile<4, 4, 10, 6, float, 40, true>;
 using F3L = Tile<4, 4, 13, 7, float, 52, true>;
 using F4L = Tile<4, 4, 16, 7, float, 64, true>;
-using D2L = Tile<4, 8, 10, 3, double, 40, true>;
-using D3L = Tile<4, 8, 13, 4, double, 52, true>;
+using D2L = Tile<4, 4, 10, 6, double, 40, true>;
+using D3L = Tile<4, 4, 13, 7, double, 52, true>;
 using D4L = Tile<4, 8, 16, 4, double, 64, true>;
 
 static_assert(F0::MAXI >= 14 && F0::MAXJ >= 5, "bin 0");

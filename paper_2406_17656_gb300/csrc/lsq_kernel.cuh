@@ -59,15 +59,16 @@
 namespace sam {
 namespace {
 
-// blocks per SM that the shared memory of a tile allows (1..4; 1..3 for the
-// FP64 tiles, whose registers do not fit 128 per thread without spilling):
+// blocks per SM that the shared memory of a tile allows (1..4; for the FP64
+// tiles, whose registers do not fit 128 per thread without spilling, 1..3, and
+// 1..2 for those of 64 slots or more, which take up to 255):
 // the register budget is held to the same count, so registers never lower
 // the occupancy that shared memory permits
 template <class TL>
 struct MinBlocks {
     static constexpr int bytes = (int)sizeof(ProbSmem<TL>) * TL::PPW * kWarpsPerBlock + 1024;
     static constexpr int raw = 233472 / bytes;
-    static constexpr int cap = sizeof(typename TL::T) == 8 ? 3 : 4;
+    static constexpr int cap = sizeof(typename TL::T) == 8 ? (TL::RS * TL::CS >= 64 ? 2 : 3) : 4;
     static constexpr int value = raw < 1 ? 1 : (raw > cap ? cap : raw);
 };
 
