@@ -231,8 +231,8 @@ cudaError_t build_work_list(sam_handle h, int N, const uint8_t *bin, int32_t *wo
                             int32_t *ws = nullptr);
 // out[j] = bin[j] where colstat[j] == flag, else no size class
 cudaError_t flagged_bins(sam_handle h, int N, const uint8_t *bin, const int32_t *colstat, int32_t flag, uint8_t *out);
-// automatic refinement's two-step launch (refine_steps < 0): the size class of
-// every column (bin), and workspace for the flagged columns' classes (bins2,
+// the size class of every column (bin), and, for automatic refinement's
+// two-step launch (refine_steps < 0), workspace for the flagged columns' classes (bins2,
 // uint8[N]), their work list (work, int32[N]), its offsets (bin_off,
 // int32[kNumBins + 1]) and the list's counters (ws, int32[2 kNumBins])
 struct RedoLists {
@@ -242,10 +242,10 @@ struct RedoLists {
 };
 // guarded refinement: in the automatic mode, the two-step solve of the columns
 // that automatic refinement flagged (redo); then the FP64 re-solve of the
-// columns the FP32 kernel flagged (list: int32[N] workspace, list_off:
-// int32[2]), then the per-outcome column counts (counts[kAutoSteps + 1], nullable)
+// columns the FP32 kernels flagged (list: int32[N] workspace for the classes
+// 0-4, args.dense_list for the large one, list_off: int32[4], zero), then the per-outcome column counts (counts[kAutoSteps + 1], nullable)
 cudaError_t launch_refine_fallback(sam_handle h, const LsqArgs &args, int N, int32_t *list, int32_t *list_off,
-                                   int64_t *counts, const RedoLists &redo = RedoLists());
+                                   int64_t *counts, const RedoLists &redo);
 
 // Least-squares launches for every size class.
 cudaError_t launch_lsq(sam_handle h, int precision, const LsqArgs &args);
@@ -255,6 +255,8 @@ cudaError_t launch_lsq(sam_handle h, int precision, const LsqArgs &args);
 cudaError_t launch_lsq_big(sam_handle h, const LsqArgs &args, int bin, bool profile = true, bool fp32 = false);
 // one size class (the items args.item_lo/item_hi select, else all of it)
 cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int bin);
+// the FP64 re-solve of columns of the classes 0-4 (bin_off[0] .. bin_off[1] of the list)
+cudaError_t launch_lsq_fp64_resolve(sam_handle h, const LsqArgs &args);
 // FP32 + refinement with a thread per column (lsq_simt.cu): size classes whose
 // LsqArgs carry the interleaved copies (kev, kev32, lrow_t)
 cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin);

@@ -7,7 +7,7 @@
 namespace sam {
 
 cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int bin) {
-    if (bin == kBinBig && precision == SAM_FP32_REFINE && args.refine_steps != 0 && args.dense_list)
+    if (bin == kBinBig && precision == SAM_FP32_REFINE && args.refine_steps != 0)
         return launch_lsq_dense(h, args, bin);
     if (bin == kBinBig) return launch_lsq_big(h, args, bin, true, precision == SAM_FP32_REFINE);
     if (precision == SAM_FP64) return launch_lsq_fp64_bin(h, args, bin);
@@ -32,12 +32,14 @@ cudaError_t launch_lsq(sam_handle h, int precision, const LsqArgs &args) {
 }
 
 namespace {
-// the columns flagged for the FP64 re-solve, in any order, into list;
-// off[1] receives their number (off[0] = 0: the list as a work-list range);
+// the columns flagged for the FP64 re-solve, in any order: those of the large
+// class into big, the others into list; off[1] and off[3] receive their
+// numbers (off[0] = off[2] = 0: the lists as work-list ranges);
 // counts (nullable): the columns that took s = 1..kAutoSteps steps, and the
 // FP64 re-solves (per-thread counts, one shared atomic per warp)
-__global__ void __launch_bounds__(256) flag_list_kernel(int N, const int32_t *colstat, const uint8_t *used, int32_t *list,
-                                                        int32_t *off, unsigned long long *counts) {
+__global__ void __launch_bounds__(256) flag_list_kernel(int N, const int32_t *colstat, const uint8_t *used,
+                                                        const uint8_t *bin, int32_t *list, int32_t *big, int32_t *off,
+                                                        unsigned long long *counts) {
     __shared__ unsigned sh[kAutoSteps + 1];
     if (threadIdx.x <= kAutoSteps) sh[threadIdx.x] = 0u;
     __syncthreads();
@@ -49,13 +51,19 @@ __global__ void __launch_bounds__(256) flag_list_kernel(int N, const int32_t *co
         const int u = counts && j < N ? used[j] : 0;
 #pragma unroll
         for (int v = 0; v <= kAutoSteps; ++v) c[v] += (u == v + 1) ? 1u : 0u;
-        const unsigned m = __ballot_sync(0xffffffffu, f);
-        if (!m) continue;
-        const int leader = __ffs(m) - 1;
-        int base = 0;
-        if (lane == leader) base = atomicAdd(&off[1], __popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (f) list[base + __popc(m & ((1u << lane) - 1u))] = (int)j;
+        if (!__any_sync(0xffffffffu, f)) continue;
+        const bool large = f && bin[j] >= kBinBig;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const bool mine = f && large == (t == 1);
+            const unsigned m = __ballot_sync(0xffffffffu, mine);
+            if (!m) continue;
+            const int leader = __ffs(m) - 1;
+            int base = 0;
+            if (lane == leader) base = atomicAdd(&off[2 * t + 1], __popc(m));
+            base = __shfl_sync(0xffffffffu, base, leader);
+            if (mine) (t ? big : list)[base + __popc(m & ((1u << lane) - 1u))] = (int)j;
+        }
     }
     if (!counts) return;
 #pragma unroll
@@ -72,12 +80,13 @@ cudaError_t launch_refine_fallback(sam_handle h, const LsqArgs &args, int N, int
                                    int64_t *counts, const RedoLists &redo) {
     cudaStream_t st = handle_stream(h);
     cudaError_t e;
+    if (!redo.bin || !args.dense_list) return cudaErrorInvalidValue;
     if (args.refine_steps < 0) {
         // automatic refinement: the columns whose first step asked for a
         // second, solved again from the start with two steps, by their size
         // classes' kernels (the guard after the second step sends a miss to
         // the FP64 re-solve below)
-        if (!redo.bin || !redo.bins2 || !redo.work || !redo.bin_off || !redo.ws) return cudaErrorInvalidValue;
+        if (!redo.bins2 || !redo.work || !redo.bin_off || !redo.ws) return cudaErrorInvalidValue;
         if ((e = flagged_bins(h, N, redo.bin, args.colstat, kStStep2, redo.bins2)) != cudaSuccess ||
             (e = build_work_list(h, N, redo.bins2, redo.work, redo.bin_off, redo.ws)) != cudaSuccess)
             return e;
@@ -95,16 +104,23 @@ cudaError_t launch_refine_fallback(sam_handle h, const LsqArgs &args, int N, int
     if (N > 0) {
         int blocks = (N + 255) / 256;
         if (blocks > handle_sms(h) * 8) blocks = handle_sms(h) * 8;
-        flag_list_kernel<<<blocks, 256, 0, st>>>(N, args.colstat, args.refine_used, list, list_off,
+        flag_list_kernel<<<blocks, 256, 0, st>>>(N, args.colstat, args.refine_used, redo.bin, list, args.dense_list,
+                                                 list_off,
                                                  reinterpret_cast<unsigned long long *>(counts));
         count_launch(h);
     }
-    // every flagged column, whatever its size class, by the FP64 kernel of
-    // the large class (results do not depend on the order of the list)
+    // the flagged columns in FP64: classes 0-4 by class 4's register tile,
+    // which holds any of them (the 3,266 such columns of sixteen 513^2 P1
+    // level-2 maps took a block of 512 threads each: patterns and maps 43.5
+    // ms, 42.3 with a warp each), the large class by its own kernel (results do not depend on the lists' order)
     LsqArgs a = args;
     a.work = list;
     a.bin_off = list_off;
     a.item_lo = a.item_hi = 0;
+    a.fac_mode = kTapeOff;  // the tape holds the FP32 factor
+    if ((e = launch_lsq_fp64_resolve(h, a)) != cudaSuccess) return e;
+    a.work = args.dense_list;
+    a.bin_off = list_off + 2;
     if ((e = launch_lsq_big(h, a, 0, false)) != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -22,13 +22,11 @@
 //   * the residual r = c - B m from its definition in FP64 (the stored
 //     entries of B, column by column), ||r||^2 plus the target's entries
 //     outside I_j.
-// Two arithmetic types.  FP64 (SAM_FP64 builds, and the re-solve of every
-// column that the refinement's guard flags): tile, QR and solves in FP64.
-// FP32 (SAM_FP32_REFINE builds): the tile, the QR and the triangular solves
-// in FP32 (half the shared memory: two blocks per SM), then the corrected
-// semi-normal-equation steps of the register classes, g = B^T r in FP64,
-// R^T R d = g in FP32, m += d, r -= B d in FP64, under the same accuracy
-// guard; a column that misses it is re-solved by the FP64 kernel.
+// Two arithmetic types.  FP64 (SAM_FP64 builds, and the re-solve of the large
+// columns that the refinement's guard flags): tile, QR and solves in FP64.
+// FP32 (SAM_FP32_REFINE builds without refinement steps): the tile, the QR and
+// the triangular solves in FP32 (half the shared memory: two blocks per SM).
+// Refined FP32 builds take lsq_dense.cu.
 #include <cfloat>
 #include <climits>
 
@@ -40,8 +38,7 @@ namespace {
 constexpr int kBigThreads = 512;
 constexpr int kBigWarps = kBigThreads / 32;
 
-enum { kSOut2 = 0, kSRes2, kSKap2, kSMsq, kSDprev, kSNum };
-enum { kRStop = 0, kRMiss, kRUsed, kRNum };
+enum { kSOut2 = 0, kSRes2, kSNum };
 
 struct __align__(16) BigHdr {
     long long colA[kBigJCap];  // value offset of column c of B (this map's values)
@@ -61,9 +58,7 @@ struct __align__(16) BigHdr {
     double y[kBigJCap];        // (Q^T c)(1:|J|), in the tile's type
     double m[kBigJCap];        // the solution
     double g[kBigJCap];        // refinement: B^T r (rounded to FP32)
-    float dv[kBigJCap];        // refinement: the correction d
     int wsum[kBigWarps];
-    int rstate[kRNum];         // refinement: stop, guard missed, steps taken
     double qp[2][4];           // reflectors k and k + 1: u_k, tau', beta (in the tile's type)
     double scal[kSNum];
     int status;                // of the current column (uniform after a barrier)
@@ -359,10 +354,10 @@ __global__ void __launch_bounds__(kBigThreads, BigBlocks<TT>::value) lsq_big_ker
         const int ld = nI;
         TT *yT = reinterpret_cast<TT *>(H.y);
         // FP32 tile: the local row of every stored entry of B, kept after the
-        // tile when it fits there (the refinement passes then skip the row
+        // tile when it fits there (the residual pass then skips the row
         // searches); lr[H.cb[c] + e] for entry e of column c
         // and their FP64 values after those (8-byte aligned): no global loads
-        // in the passes
+        // in the pass
         int *lr = reinterpret_cast<int *>(T + (size_t)ld * (nJ + 1));
         const bool keep_lr = F32 && H.status == kStOk && 3 * (int64_t)H.cb[nJ] + 1 + (int64_t)ld * (nJ + 1) <= kBigTileDoubles;
         double *bv = reinterpret_cast<double *>(lr + ((ld * (nJ + 1) + (keep_lr ? H.cb[nJ] : 0)) & 1) + (keep_lr ? H.cb[nJ] : 0));
@@ -537,128 +532,12 @@ __global__ void __launch_bounds__(kBigThreads, BigBlocks<TT>::value) lsq_big_ker
             }
             if (lane == 0 && st != kStOk) set_status(H, st);
         }
-        if (tid == 0) {
-            H.rstate[kRMiss] = 0;
-            H.rstate[kRUsed] = kAutoSteps + 1;  // solved in FP64
-        }
         __syncthreads();
         if constexpr (ADJ) {
             big_adjoint(args, H, reinterpret_cast<double *>(T), ld, nI, nJ, jj, jb, poff, args.zbig ? jj : jl,
                         zro, args.zbig ? 0 : (int64_t)kmap * args.znnz, tid, lane, warp);
             __syncthreads();  // the next column reuses the shared memory
             continue;
-        }
-        // ---- FP32 tile: corrected semi-normal-equation steps, r = c - B m0 above
-        if constexpr (F32) {
-            const bool autoref = args.refine_steps < 0;
-            const int steps = autoref ? kAutoSteps : args.refine_steps;
-            if (H.status == kStOk && steps > 0) {
-                float *gf = reinterpret_cast<float *>(H.g);
-                if (tid == 0) {  // the guard's kappa estimate (|R_kk| range) and |m_0|^2
-                    float rmax = 0.f, rmin = FLT_MAX;
-                    double m2 = 0.0;
-                    for (int k = 0; k < nJ; ++k) {
-                        const float a = fabsf((float)T[k + ld * k]);
-                        rmax = fmaxf(rmax, a);
-                        rmin = fminf(rmin, a);
-                        m2 = fma(H.m[k], H.m[k], m2);
-                    }
-                    const float kap = rmax / rmin;
-                    H.scal[kSKap2] = kap * kap;
-                    H.scal[kSMsq] = m2;
-                    H.rstate[kRStop] = 0;
-                }
-                __syncthreads();
-                for (int step = 0; step < steps; ++step) {
-                    // g = B^T r (FP64), a warp per column
-                    for (int c = warp; c < nJ; c += kBigWarps) {
-                        double acc = 0.0;
-                        for (int e = lane; e < H.clen[c]; e += 32) {
-                            const int p = keep_lr ? lr[H.cb[c] + e] : search_rows(H.I, nI, args.kri[H.kcol[c] + e]);
-                            const double b = keep_lr ? bv[H.cb[c] + e] : args.kcv[H.colA[c] + e];
-                            if (p >= 0) acc = fma(b, H.r[p], acc);
-                        }
-                        acc = warp_sum_f64(acc);
-                        if (lane == 0) gf[c] = (float)acc;  // the FP32 solve's right-hand side
-                    }
-                    __syncthreads();
-                    if (warp == 0) {
-                        // R^T y = g, then R d = y (FP32; R in the tile's upper triangle)
-                        for (int k = 0; k < nJ; ++k) {
-                            float sk = 0.f;
-                            for (int i = lane; i < k; i += 32) sk = fmaf((float)T[i + ld * k], H.dv[i], sk);
-                            sk = warp_sum<float>(sk);
-                            if (lane == 0) H.dv[k] = (gf[k] - sk) / (float)T[k + ld * k];
-                            __syncwarp();
-                        }
-                        for (int k = nJ - 1; k >= 0; --k) {
-                            const float dk = H.dv[k] / (float)T[k + ld * k];
-                            __syncwarp();
-                            for (int i = lane; i < k; i += 32) H.dv[i] = fmaf(-(float)T[i + ld * k], dk, H.dv[i]);
-                            if (lane == 0) H.dv[k] = dk;
-                            __syncwarp();
-                        }
-                        // m += d (FP64), r -= B d (FP64, column by column)
-                        float dsq = 0.f;
-                        for (int c = lane; c < nJ; c += 32) {
-                            const float d = H.dv[c];
-                            const double dd = (double)d;
-                            H.m[c] += dd;
-                            H.y[c] = dd;  // d in FP64 for r -= B d
-                            dsq = fmaf(d, d, dsq);
-                        }
-                        __syncwarp();
-                        dsq = warp_sum<float>(dsq);
-                        for (int c = 0; c < nJ; ++c) {
-                            const double dc = H.y[c];
-                            for (int e = lane; e < H.clen[c]; e += 32) {
-                                const int p = keep_lr ? lr[H.cb[c] + e] : search_rows(H.I, nI, args.kri[H.kcol[c] + e]);
-                                const double b = keep_lr ? bv[H.cb[c] + e] : args.kcv[H.colA[c] + e];
-                                if (p >= 0) H.r[p] = fma(-b, dc, H.r[p]);
-                            }
-                            __syncwarp();
-                        }
-                        if (lane == 0) {
-                            // the register classes' accuracy guard (lsq.cu), on the whole column
-                            constexpr float kTol = (float)kFallbackTol, kTol2 = kTol * kTol, kC = (float)kAutoC;
-                            const float msq = (float)H.scal[kSMsq];
-                            const float rk = (float)(kRhoSafety * kU32) * (float)H.scal[kSKap2];
-                            bool miss = !(rk < 0.5f) || rk * rk * dsq > kTol2 * (1.f - rk) * (1.f - rk) * msq;
-                            if (step == 0) {
-                                miss = miss || 4.f * kC * kC * dsq >= msq || 2.f * kC * dsq > kTol * msq;
-                            } else if (dsq > (float)kNoise2 * msq) {
-                                const float dprev2 = (float)H.scal[kSDprev];
-                                miss = miss || 4.f * dsq >= dprev2 || 4.f * dsq * dsq > kTol2 * msq * dprev2;
-                            }
-                            H.scal[kSDprev] = dsq;
-                            H.rstate[kRUsed] = step + 1;
-                            if (autoref) {
-                                if (step == 0 && !(kC * dsq > (float)kAutoTol * msq || miss)) H.rstate[kRStop] = 1;
-                                if (step == steps - 1) H.rstate[kRMiss] = miss ? 1 : 0;
-                            } else if (step == steps - 1) {
-                                H.rstate[kRMiss] = miss ? 1 : 0;
-                            }
-                        }
-                    }
-                    __syncthreads();
-                    if (H.rstate[kRStop]) break;
-                }
-                // the final residual and the solution's finiteness
-                if (warp == 0) {
-                    double s2 = 0.0;
-                    int nf = 0;
-                    for (int i = lane; i < nI; i += 32) s2 = fma(H.r[i], H.r[i], s2);
-                    for (int c = lane; c < nJ; c += 32) nf |= !isfinite(H.m[c]);
-                    s2 = warp_sum_f64(s2);
-                    nf = __any_sync(0xffffffffu, nf);
-                    if (lane == 0) {
-                        H.scal[kSRes2] = s2;
-                        if (nf || !isfinite(s2)) set_status(H, kStNonfinite);
-                        else if (H.rstate[kRMiss]) set_status(H, kStRefine);  // re-solved by the FP64 kernel
-                    }
-                }
-                __syncthreads();
-            }
         }
         // ---- outputs
         if (warp == 0) {
@@ -670,8 +549,7 @@ __global__ void __launch_bounds__(kBigThreads, BigBlocks<TT>::value) lsq_big_ker
                 const double r2 = H.scal[kSRes2];
                 args.colres[jj] = ok ? (r2 > 0.0 ? r2 : 0.0) + H.scal[kSOut2] : 0.0;
                 args.colstat[jj] = status;
-                if (args.refine_used)
-                    args.refine_used[jj] = (uint8_t)(status == kStRefine ? kAutoSteps + 1 : H.rstate[kRUsed]);
+                if (args.refine_used) args.refine_used[jj] = kAutoSteps + 1;  // a re-solve
             }
         }
         __syncthreads();  // the next column reuses the shared memory
