@@ -1377,10 +1377,20 @@ struct SimtCopies {
         a.ell_w = W;
     }
 };
-// columns from which a refined FP32 build goes to the thread-per-column kernel
-// and the most unknowns per column on average (its copies pay only where
-// nearly every column is in its size classes)
-constexpr int64_t kSimtMinColumns = 1 << 15, kSimtMeanUnknowns = 9;
+// Columns from which a refined FP32 build goes to the thread-per-column kernel,
+// where several maps share one structure (its copies of the structure are made
+// once) and where every column has its own, and the most unknowns per column on
+// average (the copies pay only where nearly every column is in its size classes).
+// Measured, build and adjoint of level-1 maps, one step, against the register
+// tiles: one structure, 2 x 16,384 columns 1.02 times as fast, 5 x 8,100 1.07, 3 x
+// 40,000 1.18; a structure for each map, 33,000 0.84, 66,000 (build) 0.96, 100,000
+// 0.98, 260,000 1.14, a 271,000-column build 1.06; 32,768 columns of shared P1 pairs
+// 0.84 (their few ill-conditioned columns go to a launch of their own).
+constexpr int64_t kSimtMinShared = 1 << 17, kSimtMinColumns = 1 << 18, kSimtMeanUnknowns = 9;
+bool simt_wanted(int precision, int refine_steps, int64_t N, bool shared, int64_t map_nnz) {
+    return precision == SAM_FP32_REFINE && refine_steps != 0 && N >= (shared ? kSimtMinShared : kSimtMinColumns) &&
+           map_nnz <= kSimtMeanUnknowns * N;
+}
 
 sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_0, int NT, const sam_pattern *S,
                       int precision, int refine_steps, const int64_t *M_offsets, int32_t *M_row_ptr,
@@ -1491,8 +1501,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     if (!ish || !icnt || !bin || !work || !bin_off || !d_st || !d_r2 || !lrow || !zloc)
         return SAM_ERR_OOM;
     SimtCopies simt;
-    if (precision == SAM_FP32_REFINE && refine_steps != 0 && N >= kSimtMinColumns &&
-        total_nnz <= kSimtMeanUnknowns * N)
+    if (simt_wanted(precision, refine_steps, N, shared, total_nnz))
         simt.alloc(sc, maxcol, N, NS, K, n, shared);
     // shadow rows, size classes, work list
     ShadowTarget tg;
@@ -2078,7 +2087,7 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
         return SAM_ERR_OOM;
     SimtCopies simt;
     int32_t *adj_off = nullptr, *adj_list = nullptr;
-    if (precision == SAM_FP32_REFINE && refine_steps != 0 && N >= kSimtMinColumns && mtot <= kSimtMeanUnknowns * N) {
+    if (simt_wanted(precision, refine_steps, N, shared, mtot)) {
         adj_off = sc.get<int32_t>(4);
         adj_list = sc.get<int32_t>((size_t)N);
         if (adj_off && adj_list) simt.alloc(sc, maxcol, N, NS, K, n, shared);
@@ -2615,7 +2624,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     cudaMemcpyAsync(d_koff, koff.data(), sizeof(int64_t) * (K + 1), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_zoff, zoff.data(), sizeof(int64_t) * (NT + 1), cudaMemcpyHostToDevice, st);
     SimtCopies simt;
-    if (precision == SAM_FP32_REFINE && refine_steps != 0 && N >= kSimtMinColumns && total_nnz <= kSimtMeanUnknowns * N)
+    if (simt_wanted(precision, refine_steps, N, shared, total_nnz))
         simt.alloc(keep, maxcol, N, NS, K, n, shared);
     ShadowTarget tg;
     tg.zcp = zcp;

@@ -46,12 +46,12 @@ def _scaled(mats):
 
 
 CASES = {
-    "width5": lambda: (_poisson(101, 4), 1),                       # 4 x 10201
-    "width7": lambda: (W.config3(nx=21, nmat=4).mats, 1),          # 4 x 9261
-    "width9": lambda: (W.config2(nx=97, nmat=4, level=1).mats, 1),  # 4 x 9409
-    "width12": lambda: (_band11(33001, 1), 0),                     # one map, one unknown per column
-    "p1": lambda: (W.config4(ncell=105, nmat=3).mats, 1),          # separate structures
-    "scaled": lambda: (_scaled(W.config2(nx=97, nmat=4, level=1).mats), 1),
+    "width5": lambda: (_poisson(182, 4), 1),                       # 4 x 33124
+    "width7": lambda: (W.config3(nx=33, nmat=4).mats, 1),          # 4 x 35937
+    "width9": lambda: (W.config2(nx=182, nmat=4, level=1).mats, 1),  # 4 x 33124
+    "width12": lambda: (_band11(262201, 1), 0),                     # one map, one unknown per column
+    "p1": lambda: (W.config4(ncell=300, nmat=3).mats, 1),          # separate structures
+    "scaled": lambda: (_scaled(W.config2(nx=182, nmat=4, level=1).mats), 1),
 }
 
 
@@ -68,7 +68,7 @@ def test_columns_against_oracle(sam, case, steps):
 
     mats, level = CASES[case]()
     n, K = mats[0].n, len(mats)
-    assert n * K >= 32768
+    assert n * K >= 1 << 17
     with sam.Handle() as h:
         aks = [sam.Csr.from_host(m) for m in mats]
         pats = h.sam_pattern_build_batched(aks, level)
@@ -93,7 +93,7 @@ def test_zero_and_nonfinite_columns(sam):
     column problem that holds it; all others are solved."""
     import torch
 
-    mats = W.config2(nx=97, nmat=4, level=1).mats
+    mats = W.config2(nx=182, nmat=4, level=1).mats
     n, K = mats[0].n, len(mats)
     data = mats[2].data.copy()
     data[mats[2].indices == 5000] = 0.0
@@ -126,7 +126,7 @@ def test_adjoint(sam, case, steps):
 
     mats, level = CASES[case]()
     n, K = mats[0].n, len(mats)
-    assert n < 32768 <= n * K
+    assert n < 1 << 17 <= n * K
     rho = 0.5
     rng = np.random.default_rng(7)
     pat = [oracle.pattern(m, level) for m in mats]
@@ -167,7 +167,7 @@ def test_factor_tape_of_a_large_batch(sam):
     is a factor of its B^T B, and a replaying adjoint equals the recomputing one."""
     import torch
 
-    mats = W.config2(nx=97, nmat=4, level=1).mats
+    mats = W.config2(nx=182, nmat=4, level=1).mats
     n, K = mats[0].n, len(mats)
     with sam.Handle() as h:
         aks = [sam.Csr.from_host(m) for m in mats]
