@@ -256,7 +256,7 @@ cudaError_t launch_lsq_big(sam_handle h, const LsqArgs &args, int bin, bool prof
 // one size class (the items args.item_lo/item_hi select, else all of it)
 cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int bin);
 // the FP64 re-solve of columns of the classes 0-4 (bin_off[0] .. bin_off[1] of the list)
-cudaError_t launch_lsq_fp64_resolve(sam_handle h, const LsqArgs &args);
+cudaError_t launch_lsq_small_fp64(sam_handle h, const LsqArgs &args);
 // FP32 + refinement with a thread per column (lsq_simt.cu): size classes whose
 // LsqArgs carry the interleaved copies (kev, kev32, lrow_t)
 cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin);

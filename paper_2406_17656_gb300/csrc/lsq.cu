@@ -109,16 +109,17 @@ cudaError_t launch_refine_fallback(sam_handle h, const LsqArgs &args, int N, int
                                                  reinterpret_cast<unsigned long long *>(counts));
         count_launch(h);
     }
-    // the flagged columns in FP64: classes 0-4 by class 4's register tile,
-    // which holds any of them (the 3,266 such columns of sixteen 513^2 P1
-    // level-2 maps took a block of 512 threads each: patterns and maps 43.5
-    // ms, 42.3 with a warp each), the large class by its own kernel (results do not depend on the lists' order)
+    // the flagged columns in FP64, by the large class's kernel; those of the
+    // classes 0-4 in two blocks per SM instead of one, since their tiles are
+    // small (results do not depend on the lists' order).  A warp per column
+    // through class 4's register tile was faster for thousands of columns but
+    // slower by 35 us for a few, and a rule on their number would make a
+    // column's bits depend on the others.
     LsqArgs a = args;
     a.work = list;
     a.bin_off = list_off;
     a.item_lo = a.item_hi = 0;
-    a.fac_mode = kTapeOff;  // the tape holds the FP32 factor
-    if ((e = launch_lsq_fp64_resolve(h, a)) != cudaSuccess) return e;
+    if ((e = launch_lsq_small_fp64(h, a)) != cudaSuccess) return e;
     a.work = args.dense_list;
     a.bin_off = list_off + 2;
     if ((e = launch_lsq_big(h, a, 0, false)) != cudaSuccess) return e;

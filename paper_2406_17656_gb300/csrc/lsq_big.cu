@@ -22,7 +22,7 @@
 //   * the residual r = c - B m from its definition in FP64 (the stored
 //     entries of B, column by column), ||r||^2 plus the target's entries
 //     outside I_j.
-// Two arithmetic types.  FP64 (SAM_FP64 builds, and the re-solve of the large
+// Two arithmetic types.  FP64 (SAM_FP64 builds, and the re-solve of the
 // columns that the refinement's guard flags): tile, QR and solves in FP64.
 // FP32 (SAM_FP32_REFINE builds without refinement steps): the tile, the QR and
 // the triangular solves in FP32 (half the shared memory: two blocks per SM).
@@ -89,6 +89,8 @@ template <typename TT>
 struct BigBlocks {
     static constexpr int value = sizeof(TT) == 4 ? 2 : 1;
 };
+// the tile that columns of the classes 0-4 need at most (64 rows, 28 columns)
+constexpr int kSmallTile = 64 * 28;
 
 __device__ __forceinline__ int search_rows(const int *I, int nI, int key) {
     int lo = 0, hi = nI - 1;
@@ -564,6 +566,16 @@ cudaError_t launch_adjoint_big(sam_handle h, const LsqArgs &args, int bin) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<handle_sms(h), kBigThreads, smem, handle_stream(h)>>>(args, bin);
+    count_launch(h);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_lsq_small_fp64(sam_handle h, const LsqArgs &args) {
+    const size_t smem = sizeof(BigHdr) + sizeof(double) * (size_t)kSmallTile;
+    auto kern = lsq_big_kernel<double>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<handle_sms(h) * 2, kBigThreads, smem, handle_stream(h)>>>(args, 0);
     count_launch(h);
     return cudaGetLastError();
 }

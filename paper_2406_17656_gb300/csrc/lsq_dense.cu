@@ -14,8 +14,8 @@
 // Where the time goes (clock64 timers in an instrumented copy, 81 x 49 columns of
 // Q1 level-3 maps, seven blocks per SM): factorisation 28%, triangular solves 16%,
 // row index and scatter 16%, Gram matrix 9%, the FP64 passes 14%.  The
-// factorisation is one warp's for up to 52 unknowns: a 4-warp tile with a
-// block barrier per pivot issued 480 warp instructions per pivot against 90.
+// factorisation is one warp's for up to 52 unknowns: it needs no block barrier
+// per pivot, as a tile over four warps did, and repeats no warp's bookkeeping.
 // Shared memory decides the blocks per SM: the dense FP32 rows of [B c] live
 // only until G exists, then the row lists and B's FP64 values take their place.
 // 128 threads per small block: 96 cost 1%, 64 cost 23%.
@@ -643,7 +643,12 @@ cudaError_t launch_dense(sam_handle h, const LsqArgs &a, int bin, int32_t *rest,
 }  // namespace
 
 cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
-    // small columns by small blocks, each next launch those that are left
+    // Small columns by small blocks, each next launch those that are left.  The
+    // class is where most columns are when map 0 has more than 27 unknowns per
+    // column on average (the register tiles' limit); otherwise its columns are
+    // few or none, and one launch less is worth more than the middle shape (three
+    // empty launches cost small builds 10 to 15 us of 390 to 1,200).
+    const bool middle = args.map_nnz_pat > 27 * (int64_t)args.n;
     cudaError_t e;
     if (args.item_hi > 0 && (e = cudaMemsetAsync(args.dense_off, 0, sizeof(int32_t) * 4, handle_stream(h))) != cudaSuccess)
         return e;  // (a chunk of a batch: the counters are used again)
@@ -653,9 +658,12 @@ cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
     a.item_lo = a.item_hi = 0;
     a.work = args.dense_list;
     a.bin_off = args.dense_off;
-    if ((e = launch_dense<DenseMedium>(h, a, 0, args.dense_list + args.dense_cap, args.dense_off + 2)) != cudaSuccess) return e;
-    a.work = args.dense_list + args.dense_cap;
-    a.bin_off = args.dense_off + 2;
+    if (middle) {
+        if ((e = launch_dense<DenseMedium>(h, a, 0, args.dense_list + args.dense_cap, args.dense_off + 2)) != cudaSuccess)
+            return e;
+        a.work = args.dense_list + args.dense_cap;
+        a.bin_off = args.dense_off + 2;
+    }
     if ((e = launch_dense<DenseLarge>(h, a, 0, nullptr, nullptr)) != cudaSuccess) return e;
     profile_end(h, bin);
     return cudaSuccess;

@@ -15,8 +15,4 @@ cudaError_t launch_lsq_fp64_bin(sam_handle h, const LsqArgs &args, int bin) {
     }
 }
 
-cudaError_t launch_lsq_fp64_resolve(sam_handle h, const LsqArgs &args) {
-    return launch_one<D4, true>(h, args, 0, false);
-}
-
 }  // namespace sam

@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<TL>::value) lsq
 // ------------------------------------------------------------ dispatch
 
 template <class TL, bool FP64>
-cudaError_t launch_one(sam_handle h, const LsqArgs &a, int bin, bool profile = true) {
+cudaError_t launch_one(sam_handle h, const LsqArgs &a, int bin) {
     const size_t smem = sizeof(ProbSmem<TL>) * TL::PPW * kWarpsPerBlock;
     auto kern = lsq_kernel<TL, FP64>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -309,10 +309,10 @@ cudaError_t launch_one(sam_handle h, const LsqArgs &a, int bin, bool profile = t
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int grid = per_sm * handle_sms(h);
-    if (profile) profile_begin(h, bin);
+    profile_begin(h, bin);
     kern<<<grid, kWarpsPerBlock * 32, smem, handle_stream(h)>>>(a, bin);
     count_launch(h);
-    if (profile) profile_end(h, bin);
+    profile_end(h, bin);
     return cudaGetLastError();
 }
 
