@@ -65,9 +65,19 @@ enum {
 /* precision of the per-column least-squares solves */
 enum {
     SAM_FP64 = 0,        /* Householder QR, triangular solves and residuals in FP64 */
-    SAM_FP32_REFINE = 1  /* Householder QR in FP32, then `refine_steps` corrected
-                            semi-normal-equation steps with FP64 residuals */
+    SAM_FP32_REFINE = 1  /* a triangular factor R in FP32, then `refine_steps`
+                            corrected semi-normal-equation steps with FP64 residuals */
 };
+
+/*
+ * The FP32 factor is the R of a Householder QR of [B c], or the Cholesky
+ * factor of B^T B with one step more than asked for, which leaves less error:
+ * for the large class (sam_size_classes), and for classes 0 and 1 of batches
+ * of many columns (131072 of maps that share one structure, 262144 otherwise)
+ * with at most nine unknowns per column on average and short symmetric
+ * sources (level-1 maps).  Such a batch's values differ from those of a
+ * smaller one by rounding, within the same target.
+ */
 
 /*
  * refine_steps = SAM_REFINE_AUTO (SAM_FP32_REFINE only): one or two steps per
@@ -88,9 +98,9 @@ enum {
  * one-step build's, bit for bit); after the
  * last step (2 in automatic mode, s otherwise) a predicted error above
  * 1e-10 |m|, or rho >= 1/2, sends the column to an FP64 Householder
- * re-solve (the large class's FP64 kernel).  The large class's FP32 tile
- * takes the same steps under the same test.  sam_refine_stats counts the
- * outcomes.
+ * re-solve (the large class's FP64 kernel).  Where
+ * the factor is a Cholesky factor, kappa comes from its diagonal and the same
+ * test follows the added step.  sam_refine_stats counts the outcomes.
  */
 #define SAM_REFINE_AUTO (-1)
 
@@ -126,8 +136,9 @@ void sam_limits(int32_t *max_rows, int32_t *max_cols);
  * |I_j| (|J_j| + 1) <= max_tile[b]; a column that fits none is
  * SAM_ERR_UNSUPPORTED.  Classes 0..4 are register tiles with
  * FP32 or FP64 arithmetic; class 5 (SAM_NUM_SIZE_CLASSES - 1) is one thread
- * block per column with the tile in shared memory (FP64 for SAM_FP64; FP32
- * with the FP64 refinement steps and their guard for SAM_FP32_REFINE); its
+ * block per column, everything in shared memory (a Householder QR in FP64 for
+ * SAM_FP64; an FP32 Cholesky factor with the FP64 refinement steps and their
+ * guard for SAM_FP32_REFINE); its
  * adjoint (sam_build_backward) runs in FP64 for either precision.  variants[b]: tile shapes of class b
  * (sam_tune, sam_set_tile_variants).  count must be SAM_NUM_SIZE_CLASSES;
  * any output may be NULL.
@@ -444,7 +455,8 @@ sam_status sam_build_backward_batched(sam_handle h, int K, const sam_csr *A_k, c
  * upper triangle of R in the build's arithmetic type (FP32 for
  * SAM_FP32_REFINE, FP64 for SAM_FP64), rows in order, each from its
  * diagonal, in a slot of |J_j| (|J_j| + 1) / 2 elements rounded up to a
- * multiple of four; slots follow the columns of the batch in order (map k's
+ * multiple of four (where the factor is a Cholesky factor: its transpose,
+ * whose diagonal is positive); slots follow the columns of the batch in order (map k's
  * columns after map k-1's).  Columns with more than 27 unknowns have no slot
  * and columns of the large class (sam_size_classes) write nothing: their
  * adjoint always factors B again (in FP64), as do the two smallest classes,

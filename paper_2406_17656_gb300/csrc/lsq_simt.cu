@@ -10,12 +10,12 @@
 //   G = B^T B, b = B^T c, G = L L^T, m = G^{-1} b  in FP32  (error ~ rho |m|)
 // and takes one step more than the build's s steps, all with r and g in FP64.
 // On level-1 columns of Q1 diffusion rho is about 3e-7 against 1.5e-7 for the
-// QR's R, so s + 1 steps leave less error than the QR kernel's s (measured
-// against 64 bits: the same 1.5e-16 for s = 2, 3e-15 against 1e-13 for s = 1).
+// QR's R (numpy, FP32 factors of sampled columns), so s + 1 steps leave less
+// error than the QR kernel's s.
 //
 // Why a thread per column: a 25 x 9 problem has 81 entries in B and 45 in G;
-// cooperating lanes spend their time on shuffles and idle register slots
-// (lsq_kernel.cuh issues about 1,900 warp instructions per column here).  Alone,
+// cooperating lanes (lsq_kernel.cuh) spend their time on shuffles and idle
+// register slots.  Alone,
 // a thread needs no communication and keeps its state in 0.5 KB of shared
 // memory, interleaved over the warp's 32 threads so that every access is free of
 // bank conflicts whatever each thread's index.  The sparse passes read the
@@ -479,7 +479,10 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
 // from the Cholesky factor with FP64 corrections, w = B lambda and r = c - B m
 // in FP64, dL/dB in gather order.  The Cholesky factor contracts an error by
 // rho, about u_32 kappa^2 per correction; a column whose estimate of rho is above
-// kAdjRho (level-1 columns: 1e-6) goes to rest, for the QR kernel.
+// kAdjRho (level-1 columns: 1e-6) goes to rest, for the QR kernel.  As the
+// forward kernel, bound by FP64 arithmetic.  Measured with the forward kernel
+// in place: 32 pairs of 512^2, level 1, two steps, map and adjoint, 70.6 ms with
+// the QR tiles' adjoint, 49.3 ms with this one.
 constexpr float kAdjRho = 1e-5f;
 
 template <class SH, int W>
