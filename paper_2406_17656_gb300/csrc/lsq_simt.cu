@@ -35,38 +35,12 @@
 #include <type_traits>
 
 #include "lsq_core.cuh"
+#include "simt_shape.cuh"
 
 namespace sam {
 namespace {
 
-constexpr __host__ __device__ int tri(int q) { return q * (q + 1) / 2; }
-
-constexpr int kSimtWarps = 16;  // one-warp blocks per SM at most (128 registers each)
-// One column problem per lane.  Word i of a lane's shared memory is at
-// 32 i + lane, so that any index of any lane hits its own bank.
-template <int MAXI_, int MAXJ_, bool ADJ = false>
-struct SimtShape {
-    static constexpr int MAXI = MAXI_, MAXJ = MAXJ_;
-    static constexpr int ROWS = MAXI + 1;                // and the row of the padding entries
-    // rows 0..MAXJ of [G b], then of L (the adjoint's r takes their place at the end)
-    static constexpr int LMIN = ADJ && 2 * ROWS > tri(MAXJ + 1) ? 2 * ROWS : tri(MAXJ + 1);
-    static constexpr int LW = (LMIN + 3) & ~3;
-    static constexpr int RW = LW;                        // r in FP64 (2 words a row); w2 during the Gram pass
-    static constexpr int W4 = (LW - 2 * ROWS) & ~3;      // w4 (4 words a row: the end of L, and r) during the Gram pass
-    static constexpr int TAB = LW + 2 * ROWS;            // columns of J
-    static constexpr int XD = (TAB + MAXJ + 1) & ~1;     // the adjoint's FP64 vectors over J
-    static constexpr int WORDS = ADJ ? XD + 4 * MAXJ : TAB + MAXJ;
-    static_assert(MAXJ % 2 == 1 && RW % 2 == 0 && XD % 2 == 0, "shape");
-    // the row groups of four that leave w4 alone
-    static constexpr int Q4 = [] {
-        int q = 0;
-        while (q + 4 <= MAXJ + 1 && tri(q + 4) <= W4) q += 4;
-        return q;
-    }();
-    static constexpr int BYTES = 128 * WORDS;
-    static constexpr int FIT = 232448 / (BYTES + 1024);
-    static constexpr int WARPS = FIT < kSimtWarps ? FIT : kSimtWarps;  // one-warp blocks per SM
-};
+constexpr __host__ __device__ int tri(int q) { return simt_tri(q); }
 
 // W entries of one column of B: values and local rows
 template <typename T, int W>
@@ -155,16 +129,19 @@ struct Simt {
         return find_sorted(args.ish + (int64_t)js * kICap, nI, args.zri[t] + zro);
     }
 
-    // [G b] = [B c]^T B in FP32: NW columns q of [B c] at a time dense in w,
+    // [G b] = [B c]^T B in FP32: two columns q of [B c] at a time dense in w,
     // their products with every column c <= q (RHS: with c as column n)
-    template <int NW, bool RHS>
-    __device__ __forceinline__ void gram(int qbeg, int qend, float *w) {
+    template <bool RHS>
+    __device__ __forceinline__ void gram() {
+        constexpr int NW = SH::NW;
+        static_assert(NW == 2, "a row of w is one float2");
+        float *w = smem + 32 * SH::WW + NW * lane;
         for (int i = 0; i < imax; ++i)
 #pragma unroll
             for (int t = 0; t < NW; ++t) w[32 * NW * i + t] = 0.f;
 #pragma unroll
         for (int t = 0; t < NW; ++t) w[32 * NW * MAXI + t] = 0.f;
-        for (int q0 = qbeg; q0 < qend; q0 += NW) {
+        for (int q0 = 0; q0 < MAXJ + 1; q0 += NW) {
             if (q0 >= nmax + (RHS ? 1 : 0)) break;
             const int cend = min(q0 + NW, nmax);
             int rows[NW][W];
@@ -191,18 +168,9 @@ struct Simt {
                 float acc[NW] = {};
 #pragma unroll
                 for (int u = 0; u < W; ++u) {
-                    const float *wr = w + 32 * NW * e.i[u];
-                    if constexpr (NW == 4) {
-                        const float4 x = *reinterpret_cast<const float4 *>(wr);
-                        acc[0] = fmaf(e.v[u], x.x, acc[0]);
-                        acc[1] = fmaf(e.v[u], x.y, acc[1]);
-                        acc[2] = fmaf(e.v[u], x.z, acc[2]);
-                        acc[3] = fmaf(e.v[u], x.w, acc[3]);
-                    } else {
-                        const float2 x = *reinterpret_cast<const float2 *>(wr);
-                        acc[0] = fmaf(e.v[u], x.x, acc[0]);
-                        acc[1] = fmaf(e.v[u], x.y, acc[1]);
-                    }
+                    const float2 x = *reinterpret_cast<const float2 *>(w + 32 * NW * e.i[u]);
+                    acc[0] = fmaf(e.v[u], x.x, acc[0]);
+                    acc[1] = fmaf(e.v[u], x.y, acc[1]);
                 }
                 const int b = tri(q0) + c;
 #pragma unroll
@@ -224,11 +192,6 @@ struct Simt {
                     }
             }
         }
-    }
-    template <bool RHS>
-    __device__ __forceinline__ void gram_all() {
-        gram<4, RHS>(0, SH::Q4, smem + 32 * SH::W4 + 4 * lane);
-        gram<2, RHS>(SH::Q4, MAXJ + 1, smem + 32 * SH::RW + 2 * lane);
     }
 
     // G = L L^T, two rows at a time in registers (RHS: the row of b gives
@@ -382,7 +345,7 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
         const bool valid = base + lane < total;
         C.begin(work[valid ? base + lane : base]);  // (idle lanes repeat a column and write nothing)
         const int n = C.n;
-        C.template gram_all<true>();
+        C.template gram<true>();
         const double out2 = C.target(R);
         C.template factor<true>();
         const bool brk = C.brk;
@@ -494,7 +457,6 @@ __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs arg
     double *Wv = reinterpret_cast<double *>(smem_f + 32 * SH::RW) + lane;  // B lambda
     double *R = reinterpret_cast<double *>(smem_f) + lane;                 // r, once L is done with
     double *X = reinterpret_cast<double *>(smem_f + 32 * SH::XD) + lane;   // m, then lambda's column factors
-    static_assert(2 * SH::ROWS <= SH::LW, "r takes L's place");
     Simt<SH, W> C(args, smem_f, lane);
     float *S = C.S;
     const int w0 = args.bin_off[bin], total = args.bin_off[bin + 1] - w0;
@@ -504,7 +466,7 @@ __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs arg
         const bool valid = base + lane < total;
         C.begin(work[valid ? base + lane : base]);  // (idle lanes repeat a column and write nothing)
         const int n = C.n;
-        C.template gram_all<false>();
+        C.template gram<false>();
         C.template factor<false>();
         const float kap2 = C.dmax / C.dmin;
         const int xb = tri(n);
@@ -629,8 +591,8 @@ cudaError_t launch_adjoint(sam_handle h, const LsqArgs &a, int bin) {
 template <int W>
 cudaError_t launch_width(sam_handle h, const LsqArgs &args, int bin) {
     switch (bin) {
-        case 0: return launch_simt<SimtShape<14, 5>, W>(h, args, 0);
-        case 1: return launch_simt<SimtShape<26, 9>, W>(h, args, 1);
+        case 0: return launch_simt<Simt0, W>(h, args, 0);
+        case 1: return launch_simt<Simt1, W>(h, args, 1);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -663,7 +625,7 @@ __global__ void __launch_bounds__(256) simt_rows_kernel(int n, int W, const int3
         const int j = j0 + q;
         const int b = j < n ? bin[j] : kBinNone;
         if (b >= kSimtBins) continue;
-        const int pad = b == 0 ? 14 : 26;  // its shape's padding row
+        const int pad = b == 0 ? Simt0::MAXI : Simt1::MAXI;  // its shape's padding row
         const int jb = jcp[j], nj = jcp[j + 1] - jb;
         int len = 0;
         if (lane < nj) {
@@ -711,8 +673,8 @@ cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args) {
     switch (args.ell_w) {
 #define SAM_ADJ_W(WW)                                                                                          \
     case WW:                                                                                                   \
-        if ((e = launch_adjoint<SimtShape<14, 5, true>, WW>(h, args, 0)) != cudaSuccess) return e;              \
-        return launch_adjoint<SimtShape<26, 9, true>, WW>(h, args, 1);
+        if ((e = launch_adjoint<Simt0Adj, WW>(h, args, 0)) != cudaSuccess) return e;              \
+        return launch_adjoint<Simt1Adj, WW>(h, args, 1);
         SAM_ADJ_W(5)
         SAM_ADJ_W(7)
         SAM_ADJ_W(9)
