@@ -45,12 +45,12 @@ struct __align__(16) DenseHdr {
     int kcol[MAXJ];           // structure offset of column c
     unsigned short cb[MAXJ + 2];  // first entry of column c in gather order
     float inv[MAXJ];          // 1 / L_kk
-    float g[MAXJ];            // B^T r, then the correction
+    double g[MAXJ];           // B^T r
     double x[MAXJ];           // the vector of the next product B x
     double m[MAXJ];           // the solution
     double part[32];              // partial sums of the warps
     int scan[32];
-    int status, nB, lo, hi, nI, brk, redo, fallback;
+    int status, nB, lo, hi, nI, brk, redo, fallback, gexp;
     float kap2, msq, da2, dprev2;
     double out2, r2;
 };
@@ -158,7 +158,7 @@ __device__ __forceinline__ void factor_from(float (&a)[SH::RS][SH::CS], float *u
             group_sync<SH>();
             const float d = uc[kk * CP + T0];
             if (!pv.brk && !(fabsf(d) <= FLT_MAX)) pv.status = kStNonfinite;  // (past a breakdown every pivot is NaN)
-            pv.brk = pv.brk || !(d > 0.f);
+            pv.brk = pv.brk || !(d >= FLT_MIN);  // (1 / d of a subnormal d overflows: the re-solve decides)
             pv.dmax = fmaxf(pv.dmax, d);
             pv.dmin = fminf(pv.dmin, d);
             const float inv = rsqrtf(d), ninv2 = -inv * inv;
@@ -367,9 +367,15 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                     if (m >= 1) g[1] = a.y;
                     if (m >= 2) g[2] = a.z;
                     if (m >= 3) g[3] = a.w;
-                    if (c < n && 4 * k4 + 3 >= c) {  // the diagonal: a zero column is rank deficient
+                    if (c < n && 4 * k4 + 3 >= c) {
+                        // the diagonal: a column of zeros is rank deficient; one
+                        // whose squares vanish in FP32 breaks the factor down
                         const float d = c - 4 * k4 == 0 ? a.x : c - 4 * k4 == 1 ? a.y : c - 4 * k4 == 2 ? a.z : a.w;
-                        if (d == 0.f) atomicMax(&H.status, (int)kStRank);
+                        if (d == 0.f) {
+                            bool zero = true;
+                            for (int e = 0; e < len; ++e) zero = zero && D.B[(int)D.row[p0 + e] * D.ldb + c] == 0.f;
+                            if (zero) atomicMax(&H.status, (int)kStRank);
+                        }
                     }
                 }
             }
@@ -435,6 +441,7 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                 if (pv.status != kStOk) H.status = max(H.status, pv.status);
                 H.brk = pv.brk ? 1 : 0;
                 H.kap2 = pv.dmax / pv.dmin;  // a lower bound on kappa(B)^2
+                H.gexp = ((__float_as_int(pv.dmax) >> 23) & 0xff) - 127;
             }
             group_sync<SH>();
         }
@@ -543,7 +550,7 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
             rs = wsum(rs);
             if (lane == 0) H.part[warp] = rs;
             __syncthreads();
-            // g = B^T r (FP64, rounded to FP32), eight lanes per column
+            // g = B^T r (FP64), eight lanes per column
             for (int c = tid >> 3; c < ((n + 3) & ~3); c += NT / 8) {
                 double a0 = 0.0;
                 if (c < n) {
@@ -557,12 +564,24 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                 }
 #pragma unroll
                 for (int o = 1; o < 8; o <<= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-                if (c < n && (lane & 7) == 0) H.g[c] = narrow_trunc(a0);
+                if (c < n && (lane & 7) == 0) H.g[c] = a0;
             }
             __syncthreads();
             if (warp == 0) {
+                // g rounded to FP32, scaled by the power of two that takes it to
+                // the size of G's pivots: on its own g is far smaller than G
+                // (by |r| / |B|) and below FP32's range where G is not yet
+                unsigned top = 0u;
 #pragma unroll
-                for (int t = 0; t < XS; ++t) x[t] = lane + 32 * t < n ? H.g[lane + 32 * t] : 0.f;
+                for (int t = 0; t < XS; ++t) {
+                    const int c = lane + 32 * t;
+                    if (c < n) top = max(top, (unsigned)__double2hiint(H.g[c]) & 0x7fffffffu);
+                }
+                top = __reduce_max_sync(0xffffffffu, top) >> 20;
+                const int up = top == 0u || top == 0x7ffu ? 0 : min(max(H.gexp - 1 - ((int)top - 1023), -1000), 1000);
+                const double sup = __hiloint2double((1023 + up) << 20, 0), sdown = __hiloint2double((1023 - up) << 20, 0);
+#pragma unroll
+                for (int t = 0; t < XS; ++t) x[t] = lane + 32 * t < n ? narrow_trunc(H.g[lane + 32 * t] * sup) : 0.f;
                 fwd();
                 back();
                 float dsq = 0.f, dg = 0.f;
@@ -570,10 +589,12 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                 for (int t = 0; t < XS; ++t) {
                     const int c = lane + 32 * t;
                     if (c < n) {
-                        H.x[c] = widen(x[t]);
-                        H.m[c] += H.x[c];
+                        const double d = widen(x[t]) * sdown;
+                        x[t] = narrow_trunc(d);
+                        H.x[c] = d;
+                        H.m[c] += d;
                         dsq = fmaf(x[t], x[t], dsq);
-                        dg = fmaf(x[t], H.g[c], dg);
+                        dg = fmaf(x[t], narrow_trunc(H.g[c]), dg);
                     }
                 }
                 dsq = wsum(dsq);
