@@ -48,8 +48,6 @@ struct __align__(16) DenseHdr {
     double g[MAXJ];           // B^T r
     double x[MAXJ];           // the vector of the next product B x
     double m[MAXJ];           // the solution
-    double part[32];              // partial sums of the warps
-    int scan[32];
     int status, nB, lo, hi, nI, brk, redo, fallback, gexp;
     float kap2, msq, da2, dprev2;
     double out2, r2;
@@ -531,7 +529,6 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
         for (int step = 0; step <= steps; ++step) {
             __syncthreads();
             // r -= B x (FP64), a row per thread, its entries by columns
-            double rs = 0.0;
             for (int i = tid; i < nI; i += NT) {
                 double ri = D.r[i];
                 const int e1 = D.rowstart[i + 1];
@@ -545,10 +542,7 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                     }
                 }
                 D.r[i] = ri;
-                rs = fma(ri, ri, rs);
             }
-            rs = wsum(rs);
-            if (lane == 0) H.part[warp] = rs;
             __syncthreads();
             // g = B^T r (FP64), eight lanes per column
             for (int c = tid >> 3; c < ((n + 3) & ~3); c += NT / 8) {
@@ -584,7 +578,8 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                 for (int t = 0; t < XS; ++t) x[t] = lane + 32 * t < n ? narrow_trunc(H.g[lane + 32 * t] * sup) : 0.f;
                 fwd();
                 back();
-                float dsq = 0.f, dg = 0.f;
+                float dsq = 0.f;
+                double dg = 0.0;
 #pragma unroll
                 for (int t = 0; t < XS; ++t) {
                     const int c = lane + 32 * t;
@@ -594,33 +589,34 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
                         H.x[c] = d;
                         H.m[c] += d;
                         dsq = fmaf(x[t], x[t], dsq);
-                        dg = fmaf(x[t], narrow_trunc(H.g[c]), dg);
+                        dg = fma(d, H.g[c], dg);
                     }
                 }
                 dsq = wsum(dsq);
-                dg = wsum(dg);
+                constexpr float kTol = (float)kFallbackTol, kTol2 = kTol * kTol, kC = (float)kAutoC;
+                const float msq = H.msq, da2 = step == 0 ? dsq : H.da2, dprev2 = H.dprev2;
+                const float rk = (float)(kRhoSafety * kU32) * H.kap2;
+                bool miss = !(rk < 0.5f) || rk * rk * dsq > kTol2 * (1.f - rk) * (1.f - rk) * msq;
+                miss = miss || 4.f * kC * kC * da2 >= msq || 4.f * kC * kC * da2 * dsq > kTol2 * msq * msq;
+                if (step > 0 && dsq > (float)kNoise2 * msq)
+                    miss = miss || 4.f * dsq >= dprev2 || 4.f * dsq * dsq > kTol2 * msq * dprev2;
+                // automatic: the second step when the first left too much
+                const bool more = autoref && step == 1 && (kC * dsq > (float)kAutoTol * msq || miss);
+                const bool redo = step < (autoref ? 1 : steps) || more;
+                // ||r - B d||^2 = ||r||^2 - d.g (g = B^T r = G d up to rounding), by
+                // one warp: the sum's order is that of every block shape
+                double r2 = -dg;
+                if (!redo) {
+                    for (int i = lane; i < nI; i += 32) r2 = fma(D.r[i], D.r[i], r2);
+                    r2 = wsum(r2);
+                }
+                __syncwarp();
                 if (lane == 0) {
-                    constexpr float kTol = (float)kFallbackTol, kTol2 = kTol * kTol, kC = (float)kAutoC;
-                    const float msq = H.msq;
-                    if (step == 0) H.da2 = dsq;
-                    const float da2 = H.da2;
-                    const float rk = (float)(kRhoSafety * kU32) * H.kap2;
-                    bool miss = !(rk < 0.5f) || rk * rk * dsq > kTol2 * (1.f - rk) * (1.f - rk) * msq;
-                    miss = miss || 4.f * kC * kC * da2 >= msq || 4.f * kC * kC * da2 * dsq > kTol2 * msq * msq;
-                    if (step > 0 && dsq > (float)kNoise2 * msq) {
-                        const float dprev2 = H.dprev2;
-                        miss = miss || 4.f * dsq >= dprev2 || 4.f * dsq * dsq > kTol2 * msq * dprev2;
-                    }
+                    H.da2 = da2;
                     H.dprev2 = dsq;
-                    // automatic: the second step when the first left too much
-                    const bool more = autoref && step == 1 && (kC * dsq > (float)kAutoTol * msq || miss);
-                    H.redo = step < (autoref ? 1 : steps) || more;
-                    if (!H.redo) {
-                        H.fallback = H.fallback || miss;
-                        double r2 = 0.0;
-                        for (int w = 0; w < NW; ++w) r2 += H.part[w];
-                        H.r2 = r2 - widen(dg);  // ||r - B d||^2 = ||r||^2 - d.g (g = B^T r = G d up to rounding)
-                    }
+                    H.redo = redo;
+                    H.r2 = r2;
+                    if (!redo) H.fallback = H.fallback || miss;
                 }
             }
             __syncthreads();
