@@ -53,11 +53,20 @@ struct __align__(16) DenseHdr {
     double out2, r2;
 };
 
+// A column whose rows span at most this finds their ranks in a bitmap (6 bytes
+// per 32 rows of the span, 6 KB at most); past it the rows are sorted, 4 bytes
+// each, so that the footprint does not grow with the numbering (the shadow pass
+// takes at most 1024 entries there).  With the bitmap alone a permuted Q1 512^2,
+// level 3 (span 262,144), filled a block's memory with it: 141.6 ms, sorted
+// 24.9; 128^3 27-point, level 1 (span 65,700): 659 ms, sorted 214.
+constexpr int kBitmapRows = 32768;
+
 // The arrays of one column after the header; bytes() is what they take.
 struct DenseLayout {
     int nI, n, nB, words, nw, ldb;
     unsigned *bm;            // row bitmap over the span [words]
     unsigned short *pre;     // rows before each word [words]
+    int *I;                  // or (wide) the sorted rows [nI]
     unsigned *mask;          // columns present in each row [nI][nw]
     double *r;               // c, then the residual [nI]
     unsigned short *rowstart;  // [nI + 1]
@@ -67,8 +76,11 @@ struct DenseLayout {
     unsigned short *pl;      // the entries by rows: their index by columns [nB]
     unsigned char *cl;       // their column [nB]
     double *val;             // and, when there is room (vals), B's entries by columns [nB]
+    int *keys;               // (wide) and before B the entries' rows, padded to a power of two [p2]
     bool vals;
-    __device__ size_t set(unsigned char *base, int nI_, int n_, int nB_, int words_, size_t room) {
+    size_t least;            // bytes of that place without the values
+    // words = 0: wide
+    __device__ size_t set(unsigned char *base, int nI_, int n_, int nB_, int words_, int p2, size_t room) {
         nI = nI_, n = n_, nB = nB_, words = words_;
         nw = (n + 31) >> 5;
         ldb = ((n + 1) + 3) & ~3;
@@ -81,15 +93,18 @@ struct DenseLayout {
         r = (double *)take(sizeof(double) * nI);
         const size_t dense = sizeof(float) * (size_t)nI * ldb, v8 = sizeof(double) * (size_t)nB;
         const size_t lists = ((3 * (size_t)nB + 15) & ~(size_t)15), all = v8 + lists;
-        vals = all <= (dense > room ? dense : room);
-        const size_t need = vals ? all : lists;
-        unsigned char *u = take(need > dense ? need : dense);
+        least = dense > lists ? dense : lists;
+        if (words == 0 && least < sizeof(int) * (size_t)p2) least = sizeof(int) * (size_t)p2;
+        vals = all <= (least > room ? least : room);
+        unsigned char *u = take(vals && all > least ? all : least);
         B = (float *)u;
+        keys = (int *)u;
         pl = (unsigned short *)u;
         cl = u + 2 * nB;
         val = (double *)(u + lists);
         L = (float *)take(sizeof(float) * tri(n + 1));
-        bm = (unsigned *)take(sizeof(unsigned) * words);
+        bm = (unsigned *)take(sizeof(unsigned) * (words ? words : nI));
+        I = (int *)bm;
         pre = (unsigned short *)take(sizeof(unsigned short) * words);
         mask = (unsigned *)take(sizeof(unsigned) * nI * nw);
         rowstart = (unsigned short *)take(sizeof(unsigned short) * (nI + 1));
@@ -99,7 +114,7 @@ struct DenseLayout {
 };
 
 // One column per block of NT threads.  Columns whose arrays take more than
-// `cap` bytes (or whose rows span too far) are appended to rest for the next kernel.
+// `cap` bytes are appended to rest for the next kernel.
 // Blocks of NT threads, BLOCKS per SM.  The factorisation runs on the first GT
 // threads as a TY x TX grid over RS TY rows (G's and b) and CS TX columns.
 template <int NT_, int BLOCKS_, int GT_, int TX_, int RS_, int CS_>
@@ -262,14 +277,18 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
         __syncthreads();
         const int nB = H.nB, lo = H.lo;
         const int64_t span = (int64_t)H.hi - lo + 1;
-        const int words = (int)((span + 31) >> 5);
+        const bool wide = span > kBitmapRows;
+        const int words = wide ? 0 : (int)((span + 31) >> 5);
+        int p2 = 1;
+        if (wide)
+            while (p2 < nB) p2 <<= 1;
         DenseLayout D;
-        bool take = n <= SH::MAXJ && nI >= n && nI <= kBigICap && nB <= kBigLCap && words <= (int)cap;
+        bool take = n <= SH::MAXJ && nI >= n && nI <= kBigICap && nB <= kBigLCap;
         if (take) {
             // the values stay in shared memory when there is room for them
-            const size_t least = D.set(base, nI, n, nB, words, 0);
+            const size_t least = D.set(base, nI, n, nB, words, p2, 0);
             take = least <= cap;
-            if (take) D.set(base, nI, n, nB, words, cap - least + sizeof(float) * (size_t)nI * D.ldb);
+            if (take) D.set(base, nI, n, nB, words, p2, cap - least + D.least);
             // (a small block leaves a column whose values do not fit to the large ones)
             take = take && (D.vals || !rest);
         }
@@ -277,46 +296,92 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
             leave(jj);
             continue;
         }
-        // ---- bitmap of the rows, rows before each word
+        if (wide) {
+            // ---- the rows sorted (bitonic), each once
+            for (int c = warp; c < n; c += NW) {
+                const int a0 = H.kcol[c], p0 = H.cb[c], len = H.cb[c + 1] - p0;
+                for (int e = lane; e < len; e += 32) D.keys[p0 + e] = args.kri[a0 + e];
+            }
+            for (int q = nB + tid; q < p2; q += NT) D.keys[q] = INT_MAX;
+            __syncthreads();
+            for (int k = 2; k <= p2; k <<= 1)
+                for (int j = k >> 1; j > 0; j >>= 1) {
+                    for (int q = tid; q < p2 / 2; q += NT) {
+                        const int a = 2 * q - (q & (j - 1)), b = a + j;  // the pair's elements
+                        const int x = D.keys[a], y = D.keys[b];
+                        if ((x > y) == ((a & k) == 0)) {
+                            D.keys[a] = y;
+                            D.keys[b] = x;
+                        }
+                    }
+                    __syncthreads();
+                }
+            if (warp == 0) {
+                int run = 0;
+                for (int q0 = 0; q0 < p2; q0 += 32) {
+                    const int q = q0 + lane;
+                    const int x = q < p2 ? D.keys[q] : INT_MAX;
+                    const bool first = x != INT_MAX && (q == 0 || D.keys[q - 1] != x);
+                    const unsigned m = __ballot_sync(0xffffffffu, first);
+                    const int pos = run + __popc(m & ((1u << lane) - 1u));
+                    if (first && pos < nI) D.I[pos] = x;
+                    run += __popc(m);
+                }
+                if (lane == 0 && run != nI) H.status = kStUnsupported;  // impossible for a consistent shadow
+            }
+            __syncthreads();
+        }
         for (int w = tid; w < words; w += NT) D.bm[w] = 0u;
         for (int q = tid; q < nI * D.nw; q += NT) D.mask[q] = 0u;
         for (int q = tid; q < nI * D.ldb / 4; q += NT) reinterpret_cast<float4 *>(D.B)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int i = tid; i < nI; i += NT) D.r[i] = 0.0;
         __syncthreads();
-        for (int c = warp; c < n; c += NW) {
-            const int a0 = H.kcol[c], len = H.cb[c + 1] - H.cb[c];
-            for (int e = lane; e < len; e += 32) {
-                const int x = args.kri[a0 + e] - lo;
-                atomicOr(&D.bm[x >> 5], 1u << (x & 31));
-            }
-        }
-        __syncthreads();
-        if (warp == 0) {
-            int run = 0;
-            for (int q = 0; q < words; q += 32) {
-                const int cnt = q + lane < words ? __popc(D.bm[q + lane]) : 0;
-                int incl = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += y;
+        if (!wide) {
+            // ---- bitmap of the rows, rows before each word
+            for (int c = warp; c < n; c += NW) {
+                const int a0 = H.kcol[c], len = H.cb[c + 1] - H.cb[c];
+                for (int e = lane; e < len; e += 32) {
+                    const int x = args.kri[a0 + e] - lo;
+                    atomicOr(&D.bm[x >> 5], 1u << (x & 31));
                 }
-                if (q + lane < words) D.pre[q + lane] = (unsigned short)(run + incl - cnt);
-                run += __shfl_sync(0xffffffffu, incl, 31);
             }
-            if (lane == 0 && run != nI) H.status = kStUnsupported;  // impossible for a consistent shadow
+            __syncthreads();
+            if (warp == 0) {
+                int run = 0;
+                for (int q = 0; q < words; q += 32) {
+                    const int cnt = q + lane < words ? __popc(D.bm[q + lane]) : 0;
+                    int incl = cnt;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += y;
+                    }
+                    if (q + lane < words) D.pre[q + lane] = (unsigned short)(run + incl - cnt);
+                    run += __shfl_sync(0xffffffffu, incl, 31);
+                }
+                if (lane == 0 && run != nI) H.status = kStUnsupported;  // impossible for a consistent shadow
+            }
+            __syncthreads();
         }
-        __syncthreads();
         if (H.status != kStOk) {
             leave(jj);
             continue;
         }
-        auto rank = [&](int x) { return (int)D.pre[x >> 5] + __popc(D.bm[x >> 5] & ((1u << (x & 31)) - 1u)); };
+        // the local row of a row of the shadow; of any row, -1 when it is none
+        auto rank = [&](int row) {
+            if (wide) return find_sorted(D.I, nI, row);
+            const int x = row - lo;
+            return (int)D.pre[x >> 5] + __popc(D.bm[x >> 5] & ((1u << (x & 31)) - 1u));
+        };
+        auto find = [&](int row) {
+            const int x = row - lo;
+            return wide || (x >= 0 && x < span && ((D.bm[x >> 5] >> (x & 31)) & 1u)) ? rank(row) : -1;
+        };
         // ---- [B c] dense in FP32, local rows, row masks; c in FP64
         for (int c = warp; c < n; c += NW) {
             const int a0 = H.kcol[c], p0 = H.cb[c], len = H.cb[c + 1] - p0;
             for (int e = lane; e < len; e += 32) {
-                const int i = rank(args.kri[a0 + e] - lo);
+                const int i = rank(args.kri[a0 + e]);
                 D.row[p0 + e] = (unsigned short)i;
                 D.B[i * D.ldb + c] = args.kcv32[H.colA[c] + e];
                 atomicOr(&D.mask[i * D.nw + (c >> 5)], 1u << (c & 31));
@@ -325,11 +390,9 @@ __global__ void __launch_bounds__(SH::NT, SH::BLOCKS) lsq_dense_kernel(LsqArgs a
         if (warp == NW - 1) {
             double o2 = 0.0;
             for (int t = zb + lane; t < ze; t += 32) {
-                const int x = args.zri[t] + zro - lo;
+                const int i = find(args.zri[t] + zro);
                 const double v = args.zcv[t];
-                const bool in = x >= 0 && x < span && ((D.bm[x >> 5] >> (x & 31)) & 1u);
-                if (in) {
-                    const int i = rank(x);
+                if (i >= 0) {
                     D.r[i] = v;
                     D.B[i * D.ldb + n] = args.zcv32[t];
                 } else {
