@@ -74,8 +74,8 @@ enum {
  * factor of B^T B with one step more than asked for, which leaves less error:
  * for the large class (sam_size_classes), and for classes 0 and 1 of batches
  * of many columns (131072 of maps that share one structure, 262144 otherwise)
- * with at most nine unknowns per column on average and short symmetric
- * sources (level-1 maps).  Such a batch's values differ from those of a
+ * with at most nine unknowns per column on average and sources of at most
+ * twelve entries per column (level-1 maps).  Such a batch's values differ from those of a
  * smaller one by rounding, within the same target.
  */
 
@@ -106,7 +106,7 @@ enum {
 
 /* flag bits for sam_set_flags */
 enum {
-    SAM_FLAG_TRUSTED = 1 /* skip CSR validation of inputs */
+    SAM_FLAG_TRUSTED = 1 /* skip CSR validation of inputs (the same results, bit for bit) */
 };
 
 /* A square sparse matrix in CSR form. */

@@ -91,6 +91,10 @@ cudaError_t launch_adjoint(sam_handle h, int precision, const LsqArgs &args) {
         a.work = args.dense_list;
         a.bin_off = args.dense_off - (kSimtBins - 1);
         if ((e = launch_adjoint_f32_bin(h, a, kSimtBins - 1)) != cudaSuccess) return e;
+        a = args;
+        a.tile_gate = args.longest;
+        for (int b = 0; args.longest && b < kSimtBins; ++b)
+            if ((e = launch_adjoint_f32_bin(h, a, b)) != cudaSuccess) return e;
     }
     for (int b = args.kev ? kSimtBins : 0; b < kRegBins; ++b) {
         // with a tape the two smallest classes still recompute R: their QR

@@ -48,6 +48,7 @@ __device__ __forceinline__ void adjoint_body(const LsqArgs &args, int bin) {
     constexpr bool TAPE = TL::LEAN;
     using T = typename TL::T;
     constexpr int P = TL::P, PPW = TL::PPW, RS = TL::RS, CS = TL::CS, JQ = TL::JQ, IQ = TL::IQ;
+    if (args.tile_gate && simt_width(*args.tile_gate)) return;  // the thread-per-column kernel takes the class
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ProbSmem<TL> *probs = reinterpret_cast<ProbSmem<TL> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

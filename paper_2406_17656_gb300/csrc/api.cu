@@ -1336,8 +1336,8 @@ sam_status tape_args(sam_handle h, Scratch &sc, const PatternGroup *g, int64_t N
 }
 
 // the longest column of K structurally symmetric sources (as long as their
-// rows: mrow, of the validation), -1 when it is not known
-int longest_column(const std::vector<char> &sym, const std::vector<int32_t> &mrow, int K) {
+// rows: mrow, of the validation), -1 when the host does not know it
+int symmetric_longest(const std::vector<char> &sym, const std::vector<int32_t> &mrow, int K) {
     int m = 0;
     for (int k = 0; k < K; ++k) {
         if (!sym[k] || mrow[k] < 0) return -1;
@@ -1348,26 +1348,41 @@ int longest_column(const std::vector<char> &sym, const std::vector<int32_t> &mro
 
 // The thread-per-column kernel's interleaved copies (lsq_simt.cu) of a batch:
 // allocated when the build takes it.  Without the memory for them the build
-// runs as it does for small batches
+// runs as it does for small batches.  Where the host does not know the longest
+// source column (unsymmetric sources, a handle that skips the validation) the
+// device finds it and the kernels of the other widths return at once: no
+// synchronisation, and the same kernel, hence the same bits, as a validating
+// handle's.
 struct SimtCopies {
     double *kev = nullptr;
     float *kev32 = nullptr;
     uint8_t *lrow_t = nullptr;
+    int32_t *longest = nullptr;
     int W = 0;
     int64_t ell_map = 0;
     bool on() const { return kev != nullptr; }
     void alloc(Scratch &sc, int maxcol, int64_t N, int NS, int K, int n, bool shared) {
-        W = simt_width(maxcol);
+        W = maxcol < 0 ? kEllW : simt_width(maxcol);
         if (!W) return;
+        if (maxcol < 0 && !(longest = sc.get<int32_t>(1))) return;
         ell_map = (((int64_t)(shared ? n : N) + 31) / 32) * (32 * W);
         const size_t ell = (size_t)(ell_map * (shared ? K : 1));
         lrow_t = sc.get<uint8_t>(((size_t)NS + 31) / 32 * 32 * kLTile);
         kev32 = sc.get<float>(ell);
         if (lrow_t && kev32) kev = sc.get<double>(ell);
     }
+    cudaError_t rows(sam_handle h, int NS, const int32_t *kcp, const int32_t *jcp, const int32_t *jri, const uint8_t *bin,
+                     const uint8_t *lrow) const {
+        if (longest) {
+            cudaError_t e = cudaMemsetAsync(longest, 0, sizeof(int32_t), h->stream);
+            if (e == cudaSuccess) e = longest_column(h, NS, kcp, longest);
+            if (e != cudaSuccess) return e;
+        }
+        return simt_rows(h, NS, W, longest, kcp, jcp, jri, bin, lrow, lrow_t);
+    }
     cudaError_t values(sam_handle h, int64_t N, int K, int n, bool shared, const int32_t *kcp, int64_t map_nnz,
                        const double *kcv) const {
-        return simt_values(h, shared ? n : (int)N, shared ? K : 1, W, kcp, map_nnz, kcv, ell_map, kev, kev32);
+        return simt_values(h, shared ? n : (int)N, shared ? K : 1, W, longest, kcp, map_nnz, kcv, ell_map, kev, kev32);
     }
     void args(LsqArgs &a) const {
         a.kev = kev;
@@ -1375,6 +1390,7 @@ struct SimtCopies {
         a.lrow_t = lrow_t;
         a.ell_map = ell_map;
         a.ell_w = W;
+        a.longest = longest;
     }
 };
 // Columns from which a refined FP32 build goes to the thread-per-column kernel,
@@ -1434,7 +1450,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     if (sg.failed) return SAM_ERR_OOM;
     bool ksym = true, zsym = true;  // structurally symmetric sources / targets
     bool one_structure = false;     // every source, every target: one structure each
-    int maxcol = -1;                // the sources' longest column, -1: not known
+    int maxcol = -1;                // the sources' longest column, -1: only the device can tell
     {
         std::vector<DevCsr> all(ak);
         all.insert(all.end(), zs.begin(), zs.end());
@@ -1443,7 +1459,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         const std::vector<std::pair<int, int>> ranges{{0, K}, {K, K + NT}};
         sam_status s = validate_all(h, sc, all, &symv, K > 1 ? &ranges : nullptr, &same, &mrow);
         if (s != SAM_OK) return s;
-        maxcol = longest_column(symv, mrow, K);
+        maxcol = symmetric_longest(symv, mrow, K);
         for (size_t q = 0; q < symv.size(); ++q) (q < ak.size() ? ksym : zsym) &= symv[q] != 0;
         one_structure = K > 1 && same[0] && same[1];
     }
@@ -1511,7 +1527,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     tg.n = n;
     tg.zloc = zloc;
     if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess ||
-        (simt.on() && simt_rows(h, NS, simt.W, kcp, g->jcp, g->jri, bin, lrow, simt.lrow_t) != cudaSuccess))
+        (simt.on() && simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess))
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, d_st) != cudaSuccess))
@@ -2040,7 +2056,7 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     if (sg.failed) return SAM_ERR_OOM;
     bool ksym = true, zsym = true;  // structurally symmetric sources / targets
     bool one_structure = false;     // every source, every target: one structure each
-    int maxcol = -1;                // the sources' longest column, -1: not known
+    int maxcol = -1;                // the sources' longest column, -1: only the device can tell
     {
         std::vector<DevCsr> all(ak);
         all.insert(all.end(), zs.begin(), zs.end());
@@ -2049,7 +2065,7 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
         const std::vector<std::pair<int, int>> ranges{{0, K}, {K, 2 * K}};
         sam_status s = validate_all(h, sc, all, &symv, K > 1 ? &ranges : nullptr, &same, &mrow);
         if (s != SAM_OK) return s;
-        maxcol = longest_column(symv, mrow, K);
+        maxcol = symmetric_longest(symv, mrow, K);
         for (size_t q = 0; q < symv.size(); ++q) (q < ak.size() ? ksym : zsym) &= symv[q] != 0;
         one_structure = K > 1 && same[0] && same[1];
     }
@@ -2100,7 +2116,7 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     tg.n = n;
     tg.zloc = zloc;
     if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, colstat, nbcnt, lrow, tg) != cudaSuccess ||
-        (simt.on() && (simt_rows(h, NS, simt.W, kcp, g->jcp, g->jri, bin, lrow, simt.lrow_t) != cudaSuccess ||
+        (simt.on() && (simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess ||
                        simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess)))
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
@@ -2531,7 +2547,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     for (int k = 0; k < K; ++k) ak[k] = DevCsr{A_k[k].n, A_k[k].nnz, A_k[k].row_ptr, A_k[k].col_idx, A_k[k].val};
     bool ksym = true, zsym = true;  // structurally symmetric sources / targets
     bool one_structure = false;     // every source, every target: one structure each
-    int maxcol = -1;                // the sources' longest column, -1: not known
+    int maxcol = -1;                // the sources' longest column, -1: only the device can tell
     {
         std::vector<DevCsr> all(ak);
         all.insert(all.end(), zs.begin(), zs.end());
@@ -2540,7 +2556,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
         const std::vector<std::pair<int, int>> ranges{{0, K}, {K, K + NT}};
         sam_status s = validate_all(h, tmp, all, &symv, K > 1 ? &ranges : nullptr, &same, &mrow);
         if (s != SAM_OK) return s;
-        maxcol = longest_column(symv, mrow, K);
+        maxcol = symmetric_longest(symv, mrow, K);
         for (size_t q = 0; q < symv.size(); ++q) (q < ak.size() ? ksym : zsym) &= symv[q] != 0;
         one_structure = K > 1 && same[0] && same[1];
     }
@@ -2633,7 +2649,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     tg.n = n;
     tg.zloc = zloc;
     if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess ||
-        (simt.on() && simt_rows(h, NS, simt.W, kcp, g->jcp, g->jri, bin, lrow, simt.lrow_t) != cudaSuccess))
+        (simt.on() && simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess))
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, d_st) != cudaSuccess))

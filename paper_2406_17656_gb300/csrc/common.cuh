@@ -38,6 +38,10 @@ constexpr int kBigTileDoubles = 23 * 1024;     // max |I_j| (|J_j| + 1) (184 KB)
 constexpr int kEllW = 12;
 constexpr int kSimtBins = 2, kSimtJ = 9;  // its size classes (0 and 1) and their most unknowns
 constexpr int kLTile = kSimtJ * kEllW;
+// the copies' width for sources whose longest column is maxcol; 0: not taken
+__host__ __device__ constexpr int simt_width(int maxcol) {
+    return maxcol < 0 || maxcol > kEllW ? 0 : maxcol <= 5 ? 5 : maxcol <= 7 ? 7 : maxcol <= 9 ? 9 : kEllW;
+}
 constexpr int kZCap = 32;    // target entries per column with a precomputed local row (zloc)
 constexpr int kZOutside = 255;  // zloc value of a target entry outside the shadow rows
 constexpr int kBinNone = 255;
@@ -114,7 +118,10 @@ struct LsqArgs {
     const float *kev32;
     const uint8_t *lrow_t;
     int64_t ell_map;             // elements of one map in kev / kev32 (shadow_shared)
-    int ell_w;                   // entries kept per source column (simt_width)
+    int ell_w;                   // entries kept per source column (simt_width), where the host knows it;
+    const int32_t *longest;      // else the longest source column: every width is launched, and the
+                                 // register tiles of the same classes, and all but one return
+    const int32_t *tile_gate;    // register tiles: nothing to do when its simt_width is not 0 (or null)
     // (the adjoint: the columns the thread-per-column kernel leaves; builds:)
     // the large class of refined FP32 builds (lsq_dense.cu), or null: the columns
     // left to its second and third launch (int32[2][dense_cap]) and their numbers
@@ -267,14 +274,15 @@ cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args);
 // order: cv[kcp[c] + u + k map_nnz]; 0 past the column's end) at
 // ((c >> 5) W + u) 32 + (c & 31) plus k ell_map, for the n columns of the
 // structure of each of K maps
-cudaError_t simt_values(sam_handle h, int n, int K, int W, const int32_t *kcp, int64_t map_nnz, const double *cv,
-                        int64_t ell_map, double *kev, float *kev32);
+// (W, or the width of *longest when longest is not null, here and in simt_rows)
+cudaError_t simt_values(sam_handle h, int n, int K, int W, const int32_t *longest, const int32_t *kcp, int64_t map_nnz,
+                        const double *cv, int64_t ell_map, double *kev, float *kev32);
 // Local rows: of entry u < W of the c-th source column of map column j (its
 // lrow, or the padding row of its size class) at ((j >> 5) kLTile + c W + u) 32 + (j & 31)
-cudaError_t simt_rows(sam_handle h, int n, int W, const int32_t *kcp, const int32_t *jcp, const int32_t *jri,
-                      const uint8_t *bin, const uint8_t *lrow, uint8_t *lrow_t);
-// the width W for sources whose longest column is maxcol; 0: not taken
-int simt_width(int maxcol);
+cudaError_t simt_rows(sam_handle h, int n, int W, const int32_t *longest, const int32_t *kcp, const int32_t *jcp,
+                      const int32_t *jri, const uint8_t *bin, const uint8_t *lrow, uint8_t *lrow_t);
+// *longest = the longest of n columns (*longest zeroed by the caller)
+cudaError_t longest_column(sam_handle h, int n, const int32_t *kcp, int32_t *longest);
 // the large class by a Cholesky factor of the normal equations (lsq_dense.cu):
 // refined FP32 builds
 cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin);

@@ -76,6 +76,7 @@ template <class TL, bool FP64>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<TL>::value) lsq_kernel(LsqArgs args, int bin) {
     using T = typename TL::T;
     constexpr int P = TL::P, PPW = TL::PPW, RS = TL::RS, CS = TL::CS, JQ = TL::JQ;
+    if (args.tile_gate && simt_width(*args.tile_gate)) return;  // the thread-per-column kernel takes the class
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ProbSmem<TL> *probs = reinterpret_cast<ProbSmem<TL> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

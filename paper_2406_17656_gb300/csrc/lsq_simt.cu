@@ -31,6 +31,7 @@
 // cycles of an SM per warp instruction, about 270 of its 460 cycles per column).
 // Loading two columns ahead costs the registers of two warps per SM (2.05 ms);
 // 12 and 16 warps per SM are equal.
+#include <algorithm>
 #include <cfloat>
 #include <type_traits>
 
@@ -332,6 +333,7 @@ struct Simt {
 template <class SH, int W>
 __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, int bin) {
     constexpr int MAXJ = SH::MAXJ;
+    if (args.longest && simt_width(*args.longest) != W) return;
     extern __shared__ __align__(16) float smem_f[];
     const int lane = threadIdx.x;
     double *R = reinterpret_cast<double *>(smem_f + 32 * SH::RW) + lane;
@@ -452,6 +454,7 @@ template <class SH, int W>
 __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs args, int bin, int32_t *rest,
                                                                     int32_t *rest_off) {
     constexpr int MAXI = SH::MAXI, MAXJ = SH::MAXJ;
+    if (args.longest && simt_width(*args.longest) != W) return;
     extern __shared__ __align__(16) float smem_f[];
     const int lane = threadIdx.x;
     double *Wv = reinterpret_cast<double *>(smem_f + 32 * SH::RW) + lane;  // B lambda
@@ -597,10 +600,19 @@ cudaError_t launch_width(sam_handle h, const LsqArgs &args, int bin) {
     }
 }
 
-__global__ void simt_values_kernel(int n, int W, const int32_t *kcp, int64_t map_nnz, const double *cv, int64_t ell_map,
-                                   double *kev, float *kev32) {
+__global__ void longest_column_kernel(int n, const int32_t *kcp, int32_t *longest) {
+    int m = 0;
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
+        m = max(m, kcp[c + 1] - kcp[c]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(longest, m);
+}
+
+__global__ void simt_values_kernel(int n, int W, const int32_t *longest, const int32_t *kcp, int64_t map_nnz,
+                                   const double *cv, int64_t ell_map, double *kev, float *kev32) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
+    if (longest) W = simt_width(*longest);
     const int k = blockIdx.y;
     const int b = kcp[c], len = kcp[c + 1] - b;
     const double *v = cv + (int64_t)k * map_nnz + b;
@@ -613,12 +625,14 @@ __global__ void simt_values_kernel(int n, int W, const int32_t *kcp, int64_t map
 }
 
 // a block per 32 columns, a warp per column at a time
-__global__ void __launch_bounds__(256) simt_rows_kernel(int n, int W, const int32_t *kcp, const int32_t *jcp,
-                                                        const int32_t *jri, const uint8_t *bin, const uint8_t *lrow,
-                                                        uint8_t *lrow_t) {
+__global__ void __launch_bounds__(256) simt_rows_kernel(int n, int W, const int32_t *longest, const int32_t *kcp,
+                                                        const int32_t *jcp, const int32_t *jri, const uint8_t *bin,
+                                                        const uint8_t *lrow, uint8_t *lrow_t) {
     __shared__ __align__(4) uint8_t sh[kLTile][32];
     __shared__ int most;
     const int j0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (longest) W = simt_width(*longest);
+    if (!W) return;
     if (threadIdx.x == 0) most = 0;
     __syncthreads();
     for (int q = warp; q < 32; q += 8) {
@@ -653,11 +667,14 @@ __global__ void __launch_bounds__(256) simt_rows_kernel(int n, int W, const int3
 
 }  // namespace
 
-int simt_width(int maxcol) {
-    return maxcol < 0 || maxcol > kEllW ? 0 : maxcol <= 5 ? 5 : maxcol <= 7 ? 7 : maxcol <= 9 ? 9 : kEllW;
-}
-
 cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin) {
+    if (args.longest) {
+        cudaError_t e;
+        if ((e = launch_width<5>(h, args, bin)) != cudaSuccess || (e = launch_width<7>(h, args, bin)) != cudaSuccess ||
+            (e = launch_width<9>(h, args, bin)) != cudaSuccess)
+            return e;
+        return launch_width<kEllW>(h, args, bin);
+    }
     switch (args.ell_w) {
         case 5: return launch_width<5>(h, args, bin);
         case 7: return launch_width<7>(h, args, bin);
@@ -669,34 +686,41 @@ cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin) {
 
 // the columns left over go to dense_list, their number to dense_off[1] (from 0)
 cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args) {
-    cudaError_t e;
-    switch (args.ell_w) {
-#define SAM_ADJ_W(WW)                                                                                          \
-    case WW:                                                                                                   \
-        if ((e = launch_adjoint<Simt0Adj, WW>(h, args, 0)) != cudaSuccess) return e;              \
-        return launch_adjoint<Simt1Adj, WW>(h, args, 1);
-        SAM_ADJ_W(5)
-        SAM_ADJ_W(7)
-        SAM_ADJ_W(9)
-        SAM_ADJ_W(kEllW)
-#undef SAM_ADJ_W
-        default: return cudaErrorInvalidValue;
-    }
+    cudaError_t e = cudaErrorInvalidValue;
+    auto width = [&](auto w) {
+        constexpr int W = decltype(w)::value;
+        if (!args.longest && args.ell_w != W) return cudaSuccess;
+        if ((e = launch_adjoint<Simt0Adj, W>(h, args, 0)) == cudaSuccess) e = launch_adjoint<Simt1Adj, W>(h, args, 1);
+        return e;
+    };
+    if (width(std::integral_constant<int, 5>()) != cudaSuccess || width(std::integral_constant<int, 7>()) != cudaSuccess ||
+        width(std::integral_constant<int, 9>()) != cudaSuccess)
+        return e;
+    width(std::integral_constant<int, kEllW>());
+    return e;
 }
 
-cudaError_t simt_values(sam_handle h, int n, int K, int W, const int32_t *kcp, int64_t map_nnz, const double *cv,
-                        int64_t ell_map, double *kev, float *kev32) {
-    if (n == 0 || K == 0) return cudaSuccess;
-    simt_values_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)K), 256, 0, handle_stream(h)>>>(
-        n, W, kcp, map_nnz, cv, ell_map, kev, kev32);
+cudaError_t longest_column(sam_handle h, int n, const int32_t *kcp, int32_t *longest) {
+    if (n == 0) return cudaSuccess;
+    longest_column_kernel<<<std::min((n + 255) / 256, 4 * handle_sms(h)), 256, 0, handle_stream(h)>>>(n, kcp, longest);
     count_launch(h);
     return cudaGetLastError();
 }
 
-cudaError_t simt_rows(sam_handle h, int n, int W, const int32_t *kcp, const int32_t *jcp, const int32_t *jri,
-                      const uint8_t *bin, const uint8_t *lrow, uint8_t *lrow_t) {
+cudaError_t simt_values(sam_handle h, int n, int K, int W, const int32_t *longest, const int32_t *kcp, int64_t map_nnz,
+                        const double *cv, int64_t ell_map, double *kev, float *kev32) {
+    if (n == 0 || K == 0) return cudaSuccess;
+    simt_values_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)K), 256, 0, handle_stream(h)>>>(
+        n, W, longest, kcp, map_nnz, cv, ell_map, kev, kev32);
+    count_launch(h);
+    return cudaGetLastError();
+}
+
+cudaError_t simt_rows(sam_handle h, int n, int W, const int32_t *longest, const int32_t *kcp, const int32_t *jcp,
+                      const int32_t *jri, const uint8_t *bin, const uint8_t *lrow, uint8_t *lrow_t) {
     if (n == 0) return cudaSuccess;
-    simt_rows_kernel<<<(unsigned)((n + 31) / 32), 256, 0, handle_stream(h)>>>(n, W, kcp, jcp, jri, bin, lrow, lrow_t);
+    simt_rows_kernel<<<(unsigned)((n + 31) / 32), 256, 0, handle_stream(h)>>>(n, W, longest, kcp, jcp, jri, bin, lrow,
+                                                                             lrow_t);
     count_launch(h);
     return cudaGetLastError();
 }
