@@ -521,7 +521,9 @@ sam_status sam_tune(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_0,
  * sam_set_tile_variants / sam_get_tile_variants -- set or read the tile
  * variant per size class (count must be SAM_NUM_SIZE_CLASSES; variant 0 for
  * every class is the default of a new handle; classes 0 and 5 have only
- * variant 0).  Set: returns
+ * variant 0).  Columns that the thread-per-column kernels take (see
+ * SAM_FP32_REFINE) have no tile: the variants of classes 0 and 1 do not
+ * concern them.  Set: returns
  * SAM_ERR_INVALID_ARG, changing nothing, if a value is out of range.
  */
 sam_status sam_set_tile_variants(sam_handle h, const int *variants, int count);

@@ -42,8 +42,10 @@ struct sam_handle_t {
     int variant[sam::kNumBins] = {0};
     // bin schedule (sam_tune / sam_set_bin_schedule): identity by default
     sam::BinSchedule sched = {{0, 1, 2, 3, 4, 5}};
-    // the tuner's record of the last build's columns per size class
+    // the tuner's record of the last build's columns per size class, and
+    // whether thread-per-column kernels took its classes 0 and 1
     bool record_hist = false;
+    bool thread_columns = false;
     int32_t *h_hist = nullptr;  // pinned [kNumBins + 1] work-list offsets
     // refinement outcomes of the last guarded build (automatic, or a fixed
     // number of steps >= 1): columns per outcome, and a pinned mirror
@@ -1403,8 +1405,11 @@ struct SimtCopies {
 // 0.98, 260,000 1.14, a 271,000-column build 1.06; 32,768 columns of shared P1 pairs
 // 0.84 (their few ill-conditioned columns go to a launch of their own).
 constexpr int64_t kSimtMinShared = 1 << 17, kSimtMinColumns = 1 << 18, kSimtMeanUnknowns = 9;
-bool simt_wanted(int precision, int refine_steps, int64_t N, bool shared, int64_t map_nnz) {
-    return precision == SAM_FP32_REFINE && refine_steps != 0 && N >= (shared ? kSimtMinShared : kSimtMinColumns) &&
+bool simt_wanted(sam_handle h, int precision, int refine_steps, int64_t N, bool shared, int64_t map_nnz) {
+    // (a bin schedule may hand all of its columns to larger classes)
+    bool any = false;
+    for (int b = 0; b < kSimtBins; ++b) any = any || h->sched.to[b] < kSimtBins;
+    return any && precision == SAM_FP32_REFINE && refine_steps != 0 && N >= (shared ? kSimtMinShared : kSimtMinColumns) &&
            map_nnz <= kSimtMeanUnknowns * N;
 }
 
@@ -1517,7 +1522,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     if (!ish || !icnt || !bin || !work || !bin_off || !d_st || !d_r2 || !lrow || !zloc)
         return SAM_ERR_OOM;
     SimtCopies simt;
-    if (simt_wanted(precision, refine_steps, N, shared, total_nnz))
+    if (simt_wanted(h, precision, refine_steps, N, shared, total_nnz))
         simt.alloc(sc, maxcol, N, NS, K, n, shared);
     // shadow rows, size classes, work list
     ShadowTarget tg;
@@ -1587,6 +1592,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     LsqArgs a;
     memset(&a, 0, sizeof(a));
     if (simt.on()) simt.args(a);
+    h->thread_columns = simt.on();
     a.kcv32 = kcv32;
     a.zcv32 = zcv32;
     a.n = n;
@@ -2103,7 +2109,7 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
         return SAM_ERR_OOM;
     SimtCopies simt;
     int32_t *adj_off = nullptr, *adj_list = nullptr;
-    if (simt_wanted(precision, refine_steps, N, shared, mtot)) {
+    if (simt_wanted(h, precision, refine_steps, N, shared, mtot)) {
         adj_off = sc.get<int32_t>(4);
         adj_list = sc.get<int32_t>((size_t)N);
         if (adj_off && adj_list) simt.alloc(sc, maxcol, N, NS, K, n, shared);
@@ -2406,6 +2412,7 @@ sam_status sam_tune(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_0,
         result = trial();
         for (int b = 0; b < kNumBins && result == SAM_OK; ++b) {
             if (h->variant[b] != var || hist[b] == 0) continue;
+            if (var > 0 && b < kSimtBins && h->thread_columns) continue;  // no tile ran
             if (cls_ms[b] < best[b]) {
                 best[b] = cls_ms[b];
                 chosen[b] = var;
@@ -2640,7 +2647,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     cudaMemcpyAsync(d_koff, koff.data(), sizeof(int64_t) * (K + 1), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_zoff, zoff.data(), sizeof(int64_t) * (NT + 1), cudaMemcpyHostToDevice, st);
     SimtCopies simt;
-    if (simt_wanted(precision, refine_steps, N, shared, total_nnz))
+    if (simt_wanted(h, precision, refine_steps, N, shared, total_nnz))
         simt.alloc(keep, maxcol, N, NS, K, n, shared);
     ShadowTarget tg;
     tg.zcp = zcp;

@@ -11,15 +11,16 @@ cudaError_t launch_lsq_bin(sam_handle h, int precision, const LsqArgs &args, int
         return launch_lsq_dense(h, args, bin);
     if (bin == kBinBig) return launch_lsq_big(h, args, bin, true, precision == SAM_FP32_REFINE);
     if (precision == SAM_FP64) return launch_lsq_fp64_bin(h, args, bin);
-    // FP32 tiles: the shape of each size class comes from the handle (sam_tune)
-    const bool b = handle_variant(h, bin) != 0;
-    if (!b && bin < kSimtBins && args.kev) {
+    if (bin < kSimtBins && args.kev) {
         const cudaError_t e = launch_lsq_simt_bin(h, args, bin);
         if (e != cudaSuccess || !args.longest) return e;
         LsqArgs t = args;
+        t.kev = nullptr;
         t.tile_gate = args.longest;
-        return bin == 0 ? launch_one<F0, false>(h, t, 0) : launch_one<F1, false>(h, t, 1);
+        return launch_lsq_bin(h, precision, t, bin);
     }
+    // FP32 tiles: the shape of each size class comes from the handle (sam_tune)
+    const bool b = handle_variant(h, bin) != 0;
     switch (bin) {
         case 0: return launch_one<F0, false>(h, args, 0);
         case 1: return b ? launch_one<F1b, false>(h, args, 1) : launch_one<F1, false>(h, args, 1);

@@ -100,3 +100,25 @@ def test_columns_against_oracle(sam, case, trusted):  # noqa: F811
     have_0 = dz[k * mats[0].nnz:].cpu().numpy()
     scale = max(np.abs(want_k).max(), np.abs(want_0).max())
     assert np.abs(have_k - want_k).max() <= 1e-7 * scale and np.abs(have_0 - want_0).max() <= 1e-7 * scale
+
+
+def test_tile_variants_do_not_concern_thread_columns(sam):  # noqa: F811
+    """A handle tuned on a small batch (variant 1 of class 1) builds a large one as a
+    new handle does; the tuner, run on a large one, leaves its classes at variant 0."""
+    import torch
+
+    mats, level = LISTS["width9"]()
+    out = []
+    for variants in ([0] * 6, [0, 1, 0, 0, 0, 0]):
+        with sam.Handle() as h:
+            h.sam_set_tile_variants(variants)
+            aks = [sam.Csr.from_host(m) for m in mats]
+            pats = h.sam_pattern_build_batched(aks, level)
+            out.append(h.sam_build_batched(aks, aks[0], pats, "fp32r", 1)[3])
+            if variants[1]:
+                h.sam_tune(aks, aks[0], pats, "fp32r", 1)
+                assert list(h.sam_get_tile_variants())[:2] == [0, 0]
+            h.sam_sync()
+            for p in pats:
+                p.destroy()
+    assert torch.equal(*out)
