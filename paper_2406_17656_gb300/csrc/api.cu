@@ -193,6 +193,13 @@ struct Scratch {
         if (p) ptrs.push_back(p);
         return (T *)p;
     }
+    // gives one allocation back early
+    void drop(void *p) {
+        const auto at = std::find(ptrs.begin(), ptrs.end(), p);
+        if (!p || at == ptrs.end()) return;
+        ptrs.erase(at);
+        pool_free(h, p);
+    }
     // hand the allocations to a longer-lived owner
     std::vector<void *> release() {
         std::vector<void *> out;
@@ -1349,8 +1356,9 @@ int symmetric_longest(const std::vector<char> &sym, const std::vector<int32_t> &
 }
 
 // The thread-per-column kernel's interleaved copies (lsq_simt.cu) of a batch:
-// allocated when the build takes it.  Without the memory for them the build
-// runs as it does for small batches.  Where the host does not know the longest
+// allocated when the build takes it, after all that it cannot do without.
+// Without the memory for them the build runs as it does for small batches (in
+// the order of its work list alone it differs).  Where the host does not know the longest
 // source column (unsymmetric sources, a handle that skips the validation) the
 // device finds it and the kernels of the other widths return at once: no
 // synchronisation, and the same kernel, hence the same bits, as a validating
@@ -1366,12 +1374,17 @@ struct SimtCopies {
     void alloc(Scratch &sc, int maxcol, int64_t N, int NS, int K, int n, bool shared) {
         W = maxcol < 0 ? kEllW : simt_width(maxcol);
         if (!W) return;
-        if (maxcol < 0 && !(longest = sc.get<int32_t>(1))) return;
+        if (maxcol < 0 && !(longest = sc.get<int32_t>(1))) return;  // (the first of them: nothing to give back)
         ell_map = (((int64_t)(shared ? n : N) + 31) / 32) * (32 * W);
         const size_t ell = (size_t)(ell_map * (shared ? K : 1));
         lrow_t = sc.get<uint8_t>(((size_t)NS + 31) / 32 * 32 * kLTile);
         kev32 = sc.get<float>(ell);
         if (lrow_t && kev32) kev = sc.get<double>(ell);
+        if (kev) return;
+        sc.drop(lrow_t);
+        sc.drop(kev32);
+        sc.drop(longest);
+        longest = nullptr;
     }
     cudaError_t rows(sam_handle h, int NS, const int32_t *kcp, const int32_t *jcp, const int32_t *jri, const uint8_t *bin,
                      const uint8_t *lrow) const {
@@ -1412,6 +1425,8 @@ bool simt_wanted(sam_handle h, int precision, int refine_steps, int64_t N, bool 
     return any && precision == SAM_FP32_REFINE && refine_steps != 0 && N >= (shared ? kSimtMinShared : kSimtMinColumns) &&
            map_nnz <= kSimtMeanUnknowns * N;
 }
+// whether the sources' columns are short enough, as far as the host knows
+bool simt_columns(int maxcol) { return maxcol < 0 || simt_width(maxcol) > 0; }
 
 sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_0, int NT, const sam_pattern *S,
                       int precision, int refine_steps, const int64_t *M_offsets, int32_t *M_row_ptr,
@@ -1521,9 +1536,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     uint8_t *zloc = sc.get<uint8_t>((size_t)N * kZCap);
     if (!ish || !icnt || !bin || !work || !bin_off || !d_st || !d_r2 || !lrow || !zloc)
         return SAM_ERR_OOM;
-    SimtCopies simt;
-    if (simt_wanted(h, precision, refine_steps, N, shared, total_nnz))
-        simt.alloc(sc, maxcol, N, NS, K, n, shared);
+    const bool thread = simt_wanted(h, precision, refine_steps, N, shared, total_nnz) && simt_columns(maxcol);
     // shadow rows, size classes, work list
     ShadowTarget tg;
     tg.zcp = zcp;
@@ -1531,8 +1544,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
     tg.zbig = NT > 1 ? 1 : 0;
     tg.n = n;
     tg.zloc = zloc;
-    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess ||
-        (simt.on() && simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess))
+    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess)
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, d_st) != cudaSuccess))
@@ -1556,7 +1568,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         }
     } ev_guard{ev_bins};
     const int32_t *off0 = nullptr;
-    if ((shared ? interleaved_work_list(h, sc, K, n, bin, work, bin_off, &chunks, &off0, simt.on())
+    if ((shared ? interleaved_work_list(h, sc, K, n, bin, work, bin_off, &chunks, &off0, thread)
                 : build_work_list(h, (int)N, bin, work, bin_off)) != cudaSuccess)
         return SAM_ERR_CUDA;
     if (h->record_hist &&
@@ -1588,11 +1600,8 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         if (round_to_f32(h, kn, kcv, kcv32) != cudaSuccess || round_to_f32(h, zn, zcv, zcv32) != cudaSuccess)
             return SAM_ERR_CUDA;
     }
-    if (simt.on() && simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess) return SAM_ERR_CUDA;
     LsqArgs a;
     memset(&a, 0, sizeof(a));
-    if (simt.on()) simt.args(a);
-    h->thread_columns = simt.on();
     a.kcv32 = kcv32;
     a.zcv32 = zcv32;
     a.n = n;
@@ -1643,6 +1652,18 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         redo.ws = sc.get<int32_t>(2 * kNumBins);
         if (!redo.bins2 || !redo.work || !redo.bin_off || !redo.ws) return SAM_ERR_OOM;
     }
+    double *fro_dev = fro ? sc.get<double>((size_t)K) : nullptr;
+    double *fro_work = fro ? sc.get<double>(segmented_sum_workspace(K)) : nullptr;
+    if (fro && (!fro_dev || !fro_work)) return SAM_ERR_OOM;
+    SimtCopies simt;
+    if (thread) simt.alloc(sc, maxcol, N, NS, K, n, shared);
+    h->thread_columns = simt.on();
+    if (simt.on()) {
+        if (simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess ||
+            simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess)
+            return SAM_ERR_CUDA;
+        simt.args(a);
+    }
     if (!chunked) {
         if (launch_lsq(h, precision, a) != cudaSuccess) return SAM_ERR_CUDA;
     } else {
@@ -1688,12 +1709,7 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         return SAM_OK;
     };
     if (status_reduce(h, d_st, N, h->d_flag) != cudaSuccess) return SAM_ERR_CUDA;
-    double *fro_dev = nullptr;
-    if (fro) {
-        fro_dev = sc.get<double>((size_t)K);
-        if (!fro_dev) return SAM_ERR_OOM;
-        if (segmented_sum_f64(h, d_r2, K, n, fro_dev, false) != cudaSuccess) return SAM_ERR_CUDA;
-    }
+    if (fro && segmented_sum_f64(h, d_r2, K, n, fro_dev, false, fro_work) != cudaSuccess) return SAM_ERR_CUDA;
     if (sg.finish() != cudaSuccess) return SAM_ERR_CUDA;
     if (fro) {
         std::vector<double> f2(K);
@@ -2107,23 +2123,13 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     if (!ish || !icnt || !bin || !colstat || !nbcnt || !dB_off || !work || !bin_off || !dbase || !dzval ||
         !dak_csc || !lrow || !zloc)
         return SAM_ERR_OOM;
-    SimtCopies simt;
-    int32_t *adj_off = nullptr, *adj_list = nullptr;
-    if (simt_wanted(h, precision, refine_steps, N, shared, mtot)) {
-        adj_off = sc.get<int32_t>(4);
-        adj_list = sc.get<int32_t>((size_t)N);
-        if (adj_off && adj_list) simt.alloc(sc, maxcol, N, NS, K, n, shared);
-        if (simt.on()) cudaMemsetAsync(adj_off, 0, sizeof(int32_t) * 4, st);
-    }
     ShadowTarget tg;
     tg.zcp = zcp;
     tg.zri = zri;
     tg.zbig = 1;
     tg.n = n;
     tg.zloc = zloc;
-    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, colstat, nbcnt, lrow, tg) != cudaSuccess ||
-        (simt.on() && (simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess ||
-                       simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess)))
+    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, colstat, nbcnt, lrow, tg) != cudaSuccess)
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, colstat) != cudaSuccess || replicate_cols(h, K, n, nbcnt) != cudaSuccess))
@@ -2186,12 +2192,21 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     a.dmres = d_dmr;
     a.dbase = dbase;
     a.znnz = zn;
-    if (simt.on()) {
-        simt.args(a);
-        a.dense_list = adj_list;
-        a.dense_off = adj_off + 1;
-    }
     if ((s = tape_args(h, sc, g, N, precision, kTapeReplay, a)) != SAM_OK) return s;
+    if (simt_wanted(h, precision, refine_steps, N, shared, mtot) && simt_columns(maxcol)) {
+        SimtCopies simt;
+        int32_t *adj_off = sc.get<int32_t>(4), *adj_list = sc.get<int32_t>((size_t)N);
+        if (adj_off && adj_list) simt.alloc(sc, maxcol, N, NS, K, n, shared);
+        if (simt.on()) {
+            cudaMemsetAsync(adj_off, 0, sizeof(int32_t) * 4, st);
+            if (simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess ||
+                simt.values(h, N, K, n, shared, kcp, ak[0].nnz, kcv) != cudaSuccess)
+                return SAM_ERR_CUDA;
+            simt.args(a);
+            a.dense_list = adj_list;
+            a.dense_off = adj_off + 1;
+        }
+    }
     if (launch_adjoint(h, precision, a) != cudaSuccess) return SAM_ERR_CUDA;
     if (adjoint_reduce(h, (int)N, kcp, g->mrp, dbase, dB, dak_csc) != cudaSuccess ||
         permute_scatter_f64(h, kn, kperm, dak_csc, d_dak) != cudaSuccess ||
@@ -2646,25 +2661,25 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     cudaMemcpyAsync(d_zptr, zptr.data(), sizeof(double *) * NT, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_koff, koff.data(), sizeof(int64_t) * (K + 1), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_zoff, zoff.data(), sizeof(int64_t) * (NT + 1), cudaMemcpyHostToDevice, st);
-    SimtCopies simt;
-    if (simt_wanted(h, precision, refine_steps, N, shared, total_nnz))
-        simt.alloc(keep, maxcol, N, NS, K, n, shared);
+    const bool thread = simt_wanted(h, precision, refine_steps, N, shared, total_nnz) && simt_columns(maxcol);
     ShadowTarget tg;
     tg.zcp = zcp;
     tg.zri = zri;
     tg.zbig = NT > 1 ? 1 : 0;
     tg.n = n;
     tg.zloc = zloc;
-    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess ||
-        (simt.on() && simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess))
+    if (shadow_and_bins(h, NS, kcp, kri, g->jcp, g->jri, ish, icnt, bin, d_st, nullptr, lrow, tg) != cudaSuccess)
         return SAM_ERR_CUDA;
     if (shared && (replicate_cols(h, K, n, icnt) != cudaSuccess || replicate_cols(h, K, n, bin) != cudaSuccess ||
                    replicate_cols(h, K, n, d_st) != cudaSuccess))
         return SAM_ERR_CUDA;
-    if ((shared ? interleaved_work_list(h, tmp, K, n, bin, work, bin_off, nullptr, nullptr, simt.on())
+    if ((shared ? interleaved_work_list(h, tmp, K, n, bin, work, bin_off, nullptr, nullptr, thread)
                 : build_work_list(h, (int)N, bin, work, bin_off)) != cudaSuccess ||
         split_map_structure(h, K, n, g->mrp, g->mci, M_row_ptr, M_col_idx) != cudaSuccess)
         return SAM_ERR_CUDA;
+    SimtCopies simt;
+    if (thread) simt.alloc(keep, maxcol, N, NS, K, n, shared);
+    if (simt.on() && simt.rows(h, NS, kcp, g->jcp, g->jri, bin, lrow) != cudaSuccess) return SAM_ERR_CUDA;
     // shadow failures (rank / unsupported) are structural: report them now
     if (status_reduce(h, d_st, N, h->d_flag) != cudaSuccess) return SAM_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return SAM_ERR_CUDA;
