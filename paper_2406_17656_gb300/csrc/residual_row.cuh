@@ -12,11 +12,17 @@ namespace sam {
 
 constexpr int kResRowBuf = 1024;  // candidate entries of one row of R a warp can hold
 
-constexpr int kResFastCnt = 768;    // candidates and bitmap words (32 columns each) up to which
-constexpr int kResFastWords = 1024;  // a row is summed through its columns' ranks
+// A row is summed through its columns' ranks where it has more candidates than a
+// warp (those take 15 rounds of the sort, less than a bitmap of any span) and at
+// most kResFastCnt, over at most kResFastWords words of 32 columns.  Per call, sort /
+// ranks: 30 candidates, 200,000 rows, over 63 words 0.593 / 0.603 ms, over 938
+// 0.591 / 0.688; 56 candidates over 129 words (32,768 rows) 0.222 / 0.186, over 969
+// (681,472 rows) 3.21 / 2.94; 234 candidates over 33 (65,536 rows) 1.11 / 0.36.
+constexpr int kResSortCnt = 32, kResFastCnt = 768;
+constexpr int kResFastWords = 1024;
 
 // ||R(i, :)||^2 for R = A_k M - A_0, computed by the calling warp.  The row's
-// entries are the products A_k(i, c) M(c, :) and -A_0(i, :).  Where their
+// entries are the products A_k(i, c) M(c, :) and -A_0(i, :).  In long rows whose
 // columns span at most 32 kResFastWords (every stencil and mesh in a banded
 // numbering), a bitmap of the columns in K gives each its rank, and the
 // products are added to V[rank] in the order of the row of A_k (the columns of
@@ -43,7 +49,7 @@ __device__ __forceinline__ double residual_row_sq(int64_t i, int lane, const int
     }
     if (cnt > kResRowBuf) return -1.0;
     const int zb = zrp[i], ze = zrp[i + 1];
-    if (cnt <= kResFastCnt) {
+    if (cnt > kResSortCnt && cnt <= kResFastCnt) {
         // the span of the columns (rows are sorted: their ends)
         int lo = INT_MAX, hi = -1;
         for (int e = krp[i] + lane; e < krp[i + 1]; e += 32) {
