@@ -725,10 +725,16 @@ cudaError_t launch_dense(sam_handle h, const LsqArgs &a, int bin, int32_t *rest,
 cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
     // Small columns by small blocks, each next launch those that are left.  The
     // class is where most columns are when map 0 has more than 27 unknowns per
-    // column on average (the register tiles' limit); otherwise its columns are
-    // few or none, and one launch less is worth more than the middle shape (three
-    // empty launches cost small builds 10 to 15 us of 390 to 1,200).
-    const bool middle = args.map_nnz_pat > 27 * (int64_t)args.n;
+    // column on average (the register tiles' limit), or more than 256 entries in
+    // the mean B (as many rows at most, where the tiles end at 64; stencils that
+    // fit the tiles have up to 225): 5 unknowns and 950 rows, 20,000 columns,
+    // 11.2 ms with the middle shape, 15.4 without.  Otherwise its columns are few or
+    // none, and one launch less is worth more (three empty launches cost small
+    // builds 10 to 15 us of 390 to 1,200).  Which shape solves a column does not
+    // change its bits.
+    const int64_t n = args.n;
+    const bool middle = args.map_nnz_pat > 27 * n ||
+                        (double)args.map_nnz_pat * (double)args.map_nnz_src > 256.0 * (double)n * (double)n;
     cudaError_t e;
     if (args.item_hi > 0 && (e = cudaMemsetAsync(args.dense_off, 0, sizeof(int32_t) * 4, handle_stream(h))) != cudaSuccess)
         return e;  // (a chunk of a batch: the counters are used again)
