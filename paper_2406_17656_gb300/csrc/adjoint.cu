@@ -85,12 +85,14 @@ cudaError_t launch_adjoint(sam_handle h, int precision, const LsqArgs &args) {
     const bool tape = args.fac_mode == kTapeReplay;
     if (args.kev) {
         // a thread per column for the smallest classes, then the columns it
-        // leaves by the larger class's QR tile
+        // leaves by their QR tiles
         if ((e = launch_adjoint_simt(h, args)) != cudaSuccess) return e;
         LsqArgs a = args;
-        a.work = args.dense_list;
-        a.bin_off = args.dense_off - (kSimtBins - 1);
-        if ((e = launch_adjoint_f32_bin(h, a, kSimtBins - 1)) != cudaSuccess) return e;
+        for (int b = 0; b < kSimtBins; ++b) {
+            a.work = args.dense_list + b * args.dense_cap;
+            a.bin_off = args.dense_off + 2 * b - b;  // (read at b and b + 1)
+            if ((e = launch_adjoint_f32_bin(h, a, b)) != cudaSuccess) return e;
+        }
         a = args;
         a.tile_gate = args.longest;
         for (int b = 0; args.longest && b < kSimtBins; ++b)

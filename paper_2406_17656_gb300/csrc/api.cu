@@ -2195,7 +2195,7 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
     if ((s = tape_args(h, sc, g, N, precision, kTapeReplay, a)) != SAM_OK) return s;
     if (simt_wanted(h, precision, refine_steps, N, shared, mtot) && simt_columns(maxcol)) {
         SimtCopies simt;
-        int32_t *adj_off = sc.get<int32_t>(4), *adj_list = sc.get<int32_t>((size_t)N);
+        int32_t *adj_off = sc.get<int32_t>(4), *adj_list = sc.get<int32_t>(kSimtBins * (size_t)N);
         if (adj_off && adj_list) simt.alloc(sc, maxcol, N, NS, K, n, shared);
         if (simt.on()) {
             cudaMemsetAsync(adj_off, 0, sizeof(int32_t) * 4, st);
@@ -2204,7 +2204,8 @@ sam_status backward_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr 
                 return SAM_ERR_CUDA;
             simt.args(a);
             a.dense_list = adj_list;
-            a.dense_off = adj_off + 1;
+            a.dense_off = adj_off;
+            a.dense_cap = N;
         }
     }
     if (launch_adjoint(h, precision, a) != cudaSuccess) return SAM_ERR_CUDA;

@@ -122,7 +122,7 @@ struct LsqArgs {
     const int32_t *longest;      // else the longest source column: every width is launched, and the
                                  // register tiles of the same classes, and all but one return
     const int32_t *tile_gate;    // register tiles: nothing to do when its simt_width is not 0 (or null)
-    // (the adjoint: the columns the thread-per-column kernel leaves; builds:)
+    // (the adjoint: the columns the thread-per-column kernel leaves, by class; builds:)
     // the large class of refined FP32 builds (lsq_dense.cu), or null: the columns
     // left to its second and third launch (int32[2][dense_cap]) and their numbers
     // as work-list ranges (int32[2][2])
@@ -267,8 +267,9 @@ cudaError_t launch_lsq_small_fp64(sam_handle h, const LsqArgs &args);
 // FP32 + refinement with a thread per column (lsq_simt.cu): size classes whose
 // LsqArgs carry the interleaved copies (kev, kev32, lrow_t)
 cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin);
-// the adjoint of its size classes; the columns it leaves to the QR kernel go to
-// args.dense_list, their number to args.dense_off[1] (zeroed by the caller)
+// the adjoint of its size classes; the columns of class b that it leaves to the QR
+// kernel go to args.dense_list + b dense_cap, their number to args.dense_off[2 b + 1]
+// (all four zeroed by the caller)
 cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args);
 // The copies of lsq_simt.cu.  Values: entry u < W of column c of map k (CSC
 // order: cv[kcp[c] + u + k map_nnz]; 0 past the column's end) at

@@ -443,12 +443,17 @@ __global__ void __launch_bounds__(32, SH::WARPS) lsq_simt_kernel(LsqArgs args, i
 // The adjoint of the columns (adjoint_core.cuh says what it computes): lambda
 // from the Cholesky factor with FP64 corrections, w = B lambda and r = c - B m
 // in FP64, dL/dB in gather order.  The Cholesky factor contracts an error by
-// rho, about u_32 kappa^2 per correction; a column whose estimate of rho is above
-// kAdjRho (level-1 columns: 1e-6) goes to rest, for the QR kernel.  As the
+// rho, about u_32 kappa^2 per correction, the QR's by half of that.  Up to rho =
+// kAdjRho one correction more than asked for (as many from two on: 1e-15 is left)
+// and past it two more leave less error than the QR kernel's; past kAdjRhoMax the
+// column goes to rest, for that kernel: a warp of such columns as soon as it has
+// its factors.  As the
 // forward kernel, bound by FP64 arithmetic.  Measured with the forward kernel
 // in place: 32 pairs of 512^2, level 1, two steps, map and adjoint, 70.6 ms with
-// the QR tiles' adjoint, 49.3 ms with this one.
-constexpr float kAdjRho = 1e-5f;
+// the QR tiles' adjoint, 49.3 ms with this one.  The adjoint of four Q1 512^2 maps,
+// two steps, QR tiles / this kernel: 7.38 / 4.53 ms; rows scaled by 10^+-1 (rho
+// around 1e-3) 7.36 / 5.26; by 10^+-3 (nearly all columns left) 7.35 / 8.19.
+constexpr float kAdjRho = 1e-5f, kAdjRhoMax = 1e-2f;
 
 template <class SH, int W>
 __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs args, int bin, int32_t *rest,
@@ -471,12 +476,19 @@ __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs arg
         const int n = C.n;
         C.template gram<false>();
         C.template factor<false>();
-        const float kap2 = C.dmax / C.dmin;
+        const float rk = (float)(kRhoSafety * kU32) * (C.dmax / C.dmin);
+        // columns that the QR kernel has to take; a warp of them is done
+        auto leave = [&] { rest[atomicAdd(&rest_off[1], 1)] = C.jj; };
+        bool left = C.status == kStOk && (C.brk || !(rk <= kAdjRhoMax));
+        if (__all_sync(0xffffffffu, left || !valid)) {
+            if (valid) leave();
+            continue;
+        }
         const int xb = tri(n);
         // ---- lambda = G^{-1} g: w = B lambda grows with it
         double gq[MAXJ], lq[MAXJ];
         float x[MAXJ];
-        float l2 = 0.f, d2 = 0.f;
+        float l2 = 0.f;
 #pragma unroll
         for (int j = 0; j < MAXJ; ++j) {
             gq[j] = (j < n && args.dmval) ? args.dmval[args.csr_pos[C.jb + j] + C.poff] : 0.0;
@@ -491,15 +503,17 @@ __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs arg
             lq[j] = widen(x[j]);
             l2 = fmaf(x[j], x[j], l2);
         }
-        const int corr = args.refine_steps < 2 ? args.refine_steps + 1 : args.refine_steps;
-        for (int step = 0; step <= corr; ++step) {
+        // this lane's corrections (past them its x is zero and changes nothing:
+        // a column's result does not depend on the warp's others)
+        int corr = args.refine_steps < 2 ? args.refine_steps + 1 : args.refine_steps;
+        for (int step = 0;; ++step) {
             C.store_x(x);
             C.add_bx(Wv, [&](int c) { return c < n ? widen(S[32 * (xb + c)]) : 0.0; });
-            if (step == corr) break;
+            if (!__any_sync(0xffffffffu, step < corr)) break;
             // correction: lambda += (L L^T)^{-1} (g - B^T w)
             C.bt_r(Wv, [&](int c, double t) { X[32 * c] = t; });
 #pragma unroll
-            for (int j = 0; j < MAXJ; ++j) x[j] = j < n ? narrow_trunc(gq[j] - X[32 * j]) : 0.f;
+            for (int j = 0; j < MAXJ; ++j) x[j] = j < n && step < corr ? narrow_trunc(gq[j] - X[32 * j]) : 0.f;
             C.fwd(x);
             C.back(x);
             float s = 0.f;
@@ -508,19 +522,20 @@ __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs arg
                 lq[j] += widen(x[j]);
                 s = fmaf(x[j], x[j], s);
             }
-            if (step == 0) d2 = s;
+            if (step == 0) {  // rho by the first correction as well, 4 |d| / |lambda|
+                left = left || (C.status == kStOk && !(16.f * s <= kAdjRhoMax * kAdjRhoMax * l2));
+                if (!(rk <= kAdjRho) || !(16.f * s <= kAdjRho * kAdjRho * l2)) corr = args.refine_steps + 2;
+                if (left) corr = 0;
+            }
         }
-        // ---- does the QR kernel have to take the column?
-        const float rk = (float)(kRhoSafety * kU32) * kap2;
-        bool leave = C.status == kStOk && (C.brk || !(rk <= kAdjRho) || !(16.f * d2 <= kAdjRho * kAdjRho * l2));
-        if (valid && leave) rest[atomicAdd(&rest_off[1], 1)] = C.jj;
+        if (valid && left) leave();
         // ---- r = c - B m
 #pragma unroll
         for (int j = 0; j < MAXJ; ++j)
             if (j < n) X[32 * j] = args.mval[args.csr_pos[C.jb + j] + C.poff];
         C.target(R);
         C.add_bx(R, [&](int c) { return c < n ? -X[32 * c] : 0.0; });
-        const bool write = valid && !leave && C.status == kStOk;
+        const bool write = valid && !left && C.status == kStOk;
         // ---- dL/dB(i, c) = r_i (lambda_c - 2 rho m_c) - w_i m_c, and where each column's block starts
         const int64_t blk = args.dB_off[C.jj];
 #pragma unroll
@@ -555,7 +570,7 @@ __global__ void __launch_bounds__(32, SH::WARPS) adjoint_simt_kernel(LsqArgs arg
                 args.dzval[zoff + t] = (i >= 0) ? Wv[32 * i] + 2.0 * rho * R[32 * i] : 2.0 * rho * args.zcv[t];
             }
         }
-        if (valid && !leave) args.colstat[C.jj] = C.status;
+        if (valid && !left) args.colstat[C.jj] = C.status;
     }
 }
 
@@ -586,7 +601,8 @@ cudaError_t launch_adjoint(sam_handle h, const LsqArgs &a, int bin) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    kern<<<per_sm * handle_sms(h), 32, smem, handle_stream(h)>>>(a, bin, a.dense_list, a.dense_off);
+    kern<<<per_sm * handle_sms(h), 32, smem, handle_stream(h)>>>(a, bin, a.dense_list + bin * a.dense_cap,
+                                                                      a.dense_off + 2 * bin);
     count_launch(h);
     return cudaGetLastError();
 }
@@ -684,7 +700,8 @@ cudaError_t launch_lsq_simt_bin(sam_handle h, const LsqArgs &args, int bin) {
     }
 }
 
-// the columns left over go to dense_list, their number to dense_off[1] (from 0)
+// the columns of class b left over go to dense_list + b dense_cap, their number
+// to dense_off[2 b + 1] (from 0)
 cudaError_t launch_adjoint_simt(sam_handle h, const LsqArgs &args) {
     cudaError_t e = cudaErrorInvalidValue;
     auto width = [&](auto w) {
