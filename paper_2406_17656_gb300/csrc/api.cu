@@ -1636,12 +1636,12 @@ sam_status build_impl(sam_handle h, int K, const sam_csr *A_k, const sam_csr *A_
         work2 = sc.get<int32_t>((size_t)N);
         a.dense_list = sc.get<int32_t>(2 * (size_t)N);
         // the counters of the large class's and the re-solve's lists, cleared together
-        a.dense_off = sc.get<int32_t>(8);
+        a.dense_off = sc.get<int32_t>(10);
         a.dense_cap = N;
-        bin_off2 = a.dense_off ? a.dense_off + 4 : nullptr;
+        bin_off2 = a.dense_off ? a.dense_off + 6 : nullptr;
         if (!a.refine_used || !work2 || !bin_off2 || !a.dense_list || !a.dense_off) return SAM_ERR_OOM;
         cudaMemsetAsync(a.refine_used, 0, (size_t)N, st);
-        cudaMemsetAsync(a.dense_off, 0, sizeof(int32_t) * 8, st);
+        cudaMemsetAsync(a.dense_off, 0, sizeof(int32_t) * 10, st);
         redo.bin = bin;
     }
     if (autoref) {
@@ -2627,8 +2627,8 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
     uint8_t *refine_used = autoref ? keep.get<uint8_t>((size_t)N) : nullptr;
     int32_t *work2 = autoref ? keep.get<int32_t>((size_t)N) : nullptr;
     int32_t *dense_list = autoref ? keep.get<int32_t>(2 * (size_t)N) : nullptr;
-    int32_t *dense_off = autoref ? keep.get<int32_t>(8) : nullptr;
-    int32_t *bin_off2 = dense_off ? dense_off + 4 : nullptr;  // cleared with them
+    int32_t *dense_off = autoref ? keep.get<int32_t>(10) : nullptr;
+    int32_t *bin_off2 = dense_off ? dense_off + 6 : nullptr;  // cleared with them
     if (autoref && (!refine_used || !work2 || !bin_off2 || !dense_list || !dense_off)) return SAM_ERR_OOM;
     // automatic refinement: the two-step launch's own lists (the first
     // launch's work list is read again at every replay)
@@ -2733,7 +2733,7 @@ sam_status sam_plan_create(sam_handle h, int K, const sam_csr *A_k, const sam_cs
                   cudaMemsetAsync(M_val, 0, sizeof(double) * (size_t)total_nnz, cs) == cudaSuccess &&
                   cudaMemsetAsync(d_r2, 0, sizeof(double) * (size_t)N, cs) == cudaSuccess &&
                   (!autoref || (cudaMemsetAsync(refine_used, 0, (size_t)N, cs) == cudaSuccess &&
-                                cudaMemsetAsync(dense_off, 0, sizeof(int32_t) * 8, cs) == cudaSuccess)) &&
+                                cudaMemsetAsync(dense_off, 0, sizeof(int32_t) * 10, cs) == cudaSuccess)) &&
                   launch_lsq(h, precision, a) == cudaSuccess &&
                   (!autoref || launch_refine_fallback(h, a, (int)N, work2, bin_off2, h->d_refine, redo) == cudaSuccess) &&
                   status_reduce(h, d_st, N, h->d_flag) == cudaSuccess &&

@@ -124,8 +124,8 @@ struct LsqArgs {
     const int32_t *tile_gate;    // register tiles: nothing to do when its simt_width is not 0 (or null)
     // (the adjoint: the columns the thread-per-column kernel leaves, by class; builds:)
     // the large class of refined FP32 builds (lsq_dense.cu), or null: the columns
-    // left to its second and third launch (int32[2][dense_cap]) and their numbers
-    // as work-list ranges (int32[2][2])
+    // left to its later launches (int32[2][dense_cap], in turn) and their numbers
+    // as work-list ranges (int32[3][2])
     int32_t *dense_list, *dense_off;
     int64_t dense_cap;
     int item_lo, item_hi;        // item_hi > 0: only items [item_lo, item_hi) of the launched class

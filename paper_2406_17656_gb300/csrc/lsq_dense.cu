@@ -128,6 +128,7 @@ struct DenseShape {
 };
 using DenseSmall = DenseShape<128, 7, 32, 4, 7, 13>;   // up to 52 unknowns
 using DenseMedium = DenseShape<128, 3, 128, 8, 9, 16>;  // up to 128
+using DenseHalf = DenseShape<256, 2, 128, 8, 9, 16>;  // up to 128
 using DenseLarge = DenseShape<512, 1, 128, 8, 9, 16>;  // up to 128
 static_assert(DenseSmall::UW % 4 == 0 && DenseLarge::UW % 4 == 0, "alignment");
 static_assert(DenseSmall::MAXJ == 52 && DenseLarge::MAXJ == kBigJCap, "shapes");
@@ -727,16 +728,17 @@ cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
     // class is where most columns are when map 0 has more than 27 unknowns per
     // column on average (the register tiles' limit), or more than 256 entries in
     // the mean B (as many rows at most, where the tiles end at 64; stencils that
-    // fit the tiles have up to 225): 5 unknowns and 950 rows, 20,000 columns,
-    // 11.2 ms with the middle shape, 15.4 without.  Otherwise its columns are few or
-    // none, and one launch less is worth more (three empty launches cost small
-    // builds 10 to 15 us of 390 to 1,200).  Which shape solves a column does not
-    // change its bits.
+    // fit the tiles have up to 225).  Then the shapes of three and two blocks per SM
+    // come between: 20,000 columns of 5 unknowns and 950 rows 11.4 ms with them,
+    // 15.4 without; of 14 unknowns and 840 rows (80 KB each) 4.7, 7.3 with three
+    // blocks per SM alone.  Otherwise the class's columns are few or none, and two
+    // launches less are worth more (three empty ones cost small builds 10 to 15 us
+    // of 390 to 1,200).  Which shape solves a column does not change its bits.
     const int64_t n = args.n;
     const bool middle = args.map_nnz_pat > 27 * n ||
                         (double)args.map_nnz_pat * (double)args.map_nnz_src > 256.0 * (double)n * (double)n;
     cudaError_t e;
-    if (args.item_hi > 0 && (e = cudaMemsetAsync(args.dense_off, 0, sizeof(int32_t) * 4, handle_stream(h))) != cudaSuccess)
+    if (args.item_hi > 0 && (e = cudaMemsetAsync(args.dense_off, 0, sizeof(int32_t) * 6, handle_stream(h))) != cudaSuccess)
         return e;  // (a chunk of a batch: the counters are used again)
     profile_begin(h, bin);
     if ((e = launch_dense<DenseSmall>(h, args, bin, args.dense_list, args.dense_off)) != cudaSuccess) return e;
@@ -745,10 +747,14 @@ cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
     a.work = args.dense_list;
     a.bin_off = args.dense_off;
     if (middle) {
+        // (the two lists in turn: what one launch leaves, the next reads)
         if ((e = launch_dense<DenseMedium>(h, a, 0, args.dense_list + args.dense_cap, args.dense_off + 2)) != cudaSuccess)
             return e;
         a.work = args.dense_list + args.dense_cap;
         a.bin_off = args.dense_off + 2;
+        if ((e = launch_dense<DenseHalf>(h, a, 0, args.dense_list, args.dense_off + 4)) != cudaSuccess) return e;
+        a.work = args.dense_list;
+        a.bin_off = args.dense_off + 4;
     }
     if ((e = launch_dense<DenseLarge>(h, a, 0, nullptr, nullptr)) != cudaSuccess) return e;
     profile_end(h, bin);
