@@ -128,7 +128,7 @@ struct DenseShape {
 };
 using DenseSmall = DenseShape<128, 7, 32, 4, 7, 13>;   // up to 52 unknowns
 using DenseMedium = DenseShape<128, 3, 128, 8, 9, 16>;  // up to 128
-using DenseHalf = DenseShape<256, 2, 128, 8, 9, 16>;  // up to 128
+using DenseHalf = DenseShape<256, 2, 32, 4, 7, 13>;    // up to 52
 using DenseLarge = DenseShape<512, 1, 128, 8, 9, 16>;  // up to 128
 static_assert(DenseSmall::UW % 4 == 0 && DenseLarge::UW % 4 == 0, "alignment");
 static_assert(DenseSmall::MAXJ == 52 && DenseLarge::MAXJ == kBigJCap, "shapes");
@@ -730,10 +730,11 @@ cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
     // the mean B (as many rows at most, where the tiles end at 64; stencils that
     // fit the tiles have up to 225).  Then the shapes of three and two blocks per SM
     // come between: 20,000 columns of 5 unknowns and 950 rows 11.4 ms with them,
-    // 15.4 without; of 14 unknowns and 840 rows (80 KB each) 4.7, 7.3 with three
+    // 15.4 without; of 14 unknowns and 840 rows (80 KB each) 4.3, 7.3 with three
     // blocks per SM alone.  Otherwise the class's columns are few or none, and two
     // launches less are worth more (three empty ones cost small builds 10 to 15 us
-    // of 390 to 1,200).  Which shape solves a column does not change its bits.
+    // of 390 to 1,200; two per SM with a handful of columns, where the mean is past
+    // its 52 unknowns, 100 us of 15.3 ms).  Which shape solves a column does not change its bits.
     const int64_t n = args.n;
     const bool middle = args.map_nnz_pat > 27 * n ||
                         (double)args.map_nnz_pat * (double)args.map_nnz_src > 256.0 * (double)n * (double)n;
@@ -752,9 +753,11 @@ cudaError_t launch_lsq_dense(sam_handle h, const LsqArgs &args, int bin) {
             return e;
         a.work = args.dense_list + args.dense_cap;
         a.bin_off = args.dense_off + 2;
-        if ((e = launch_dense<DenseHalf>(h, a, 0, args.dense_list, args.dense_off + 4)) != cudaSuccess) return e;
-        a.work = args.dense_list;
-        a.bin_off = args.dense_off + 4;
+        if (args.map_nnz_pat <= DenseHalf::MAXJ * n) {
+            if ((e = launch_dense<DenseHalf>(h, a, 0, args.dense_list, args.dense_off + 4)) != cudaSuccess) return e;
+            a.work = args.dense_list;
+            a.bin_off = args.dense_off + 4;
+        }
     }
     if ((e = launch_dense<DenseLarge>(h, a, 0, nullptr, nullptr)) != cudaSuccess) return e;
     profile_end(h, bin);
