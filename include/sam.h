@@ -76,7 +76,10 @@ enum {
  * of many columns (131072 of maps that share one structure, 262144 otherwise)
  * with at most nine unknowns per column on average and sources of at most
  * twelve entries per column (level-1 maps).  Such a batch's values differ from those of a
- * smaller one by rounding, within the same target.
+ * smaller one by rounding, within the same target: the same map built alone, or in
+ * the part of a sequence that another rank takes, agrees to the accuracy target,
+ * not bit for bit.  The adjoint of such a batch takes the Cholesky factor likewise (see
+ * sam_build_backward).
  */
 
 /*
@@ -410,7 +413,11 @@ sam_status sam_gmres_batched(sam_handle h, int K, const sam_csr *A, const sam_cs
  * A_k entry receives the sum of its contributions from all columns, added
  * in a fixed order (deterministic).  lambda uses the recomputed QR (FP32 R
  * plus `refine_steps` FP64-residual corrections for SAM_FP32_REFINE), or the
- * forward build's R from a factor tape (sam_set_factor_tape).
+ * forward build's R from a factor tape (sam_set_factor_tape).  Columns of
+ * classes 0 and 1 in batches large enough for the builds' Cholesky factor
+ * (see SAM_FP32_REFINE) take that factor and up to two corrections more, which
+ * leaves less error; their gradients differ from those of a smaller batch, or of
+ * single calls, by rounding.
  * dA_k_val[nnz(A_k)], dA_0_val[nnz(A_0)]: outputs in the CSR order of A_k
  * and A_0 (overwritten).  dM_resid (nullable, nnz(S), CSR order of the map):
  * receives w * d||A_k M - A_0||_F^2 / dM = -2 w A_k^T R on the pattern (zero

@@ -57,7 +57,7 @@ struct __align__(16) BigHdr {
     double r[kBigICap];        // c, then the residual
     double y[kBigJCap];        // (Q^T c)(1:|J|), in the tile's type
     double m[kBigJCap];        // the solution
-    double g[kBigJCap];        // refinement: B^T r (rounded to FP32)
+    double g[kBigJCap];        // the adjoint: dL/dm
     int wsum[kBigWarps];
     double qp[2][4];           // reflectors k and k + 1: u_k, tau', beta (in the tile's type)
     double scal[kSNum];

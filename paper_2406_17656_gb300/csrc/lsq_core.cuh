@@ -513,11 +513,13 @@ using F4 = Tile<4, 4, 16, 7, float, 64>;
 // cost it the same for one column problem per warp as for two: two problems of
 // 16 lanes (class 1: eight of 4 lanes, not four of 8) take 109 column slots for 25
 // unknowns where one of 32 took 73 each, and half the reflector overhead, at
-// 255 registers and 8 warps per SM, which still fill the pipe.  With the QR's
+// 255 registers and 8 warps per SM (class 2, of 60 slots: 168 registers, 12 warps
+// and 72 bytes of spills), which still fill the pipe.  With the QR's
 // shorter sums (QRPhase) two 256^2 Q1 level-2 maps went from 16.6 to 9.46 ms,
-// eight level-1 ones from 7.30 to 4.60, a level-2 map with its residual and adjoint
-// from 27.8 to 16.2.  Class 4 (16 x 7 slots: 224 registers) keeps 32 lanes,
-// with 255 registers instead of 168 and 476 bytes of spills.
+// two 5-point ones (class 2) from 7.29 to 4.46, eight level-1 ones from 7.30 to 4.60, a
+// level-2 map with its residual and adjoint from 27.8 to 16.2.  Class 4 keeps 32
+// lanes (16 would hold 16 x 7 slots, 224 registers of tile alone), at 252 registers
+// without spills instead of 168 with 476 bytes of them.
 using D0 = Tile<2, 2, 7, 3, double, 14>;
 using D1 = Tile<2, 2, 13, 5, double, 26>;
 using D2 = Tile<4, 4, 10, 6, double, 40, false, true>;
@@ -530,7 +532,9 @@ using F2b = Tile<4, 8, 10, 3, float, 40, false, true>;
 using F3b = Tile<4, 8, 13, 4, float, 52, false, true>;
 using F4b = Tile<4, 8, 16, 4, float, 64>;
 // the adjoint's shapes when R comes from a factor tape (size classes 2-4;
-// the two smallest recompute their small QR)
+// the two smallest recompute their small QR).  The FP64 ones have the solves' lanes:
+// two 5-point level-2 maps of 256^2 1.74 -> 1.36 ms against 32 lanes, 9-point 2.39 ->
+// 2.05 (calls of 2,000 columns 2% slower), though they spill 100 and 80 bytes
 using F2L = Tile<4, 4, 10, 6, float, 40, true>;
 using F3L = Tile<4, 4, 13, 7, float, 52, true>;
 using F4L = Tile<4, 4, 16, 7, float, 64, true>;

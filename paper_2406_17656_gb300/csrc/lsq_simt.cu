@@ -26,9 +26,13 @@
 // per SM, whose latency nothing hides (measured 1.6 times slower than the QR
 // kernel on 49 x 25 columns), so they keep lsq_kernel.cuh.
 //
-// Measured, 4 maps of 512^2 unknowns, level 1, two steps: 1.65 ms for the class-1
-// launch against 3.94 ms (lsq_kernel.cuh); FP64 arithmetic bounds it (16
-// cycles of an SM per warp instruction, about 270 of its 460 cycles per column).
+// Measured, 4 maps of 512^2 unknowns, level 1, two steps: 1.83 ms for the class-1
+// launch against 3.91 ms (lsq_kernel.cuh).  FP64 arithmetic bounds it: the pipe is
+// active in 58% of the cycles (16 of them per warp instruction) at 13 warps per SM,
+// which wait for the operands of the FP64 passes (shared memory pipe 48%; 17,100
+// warp instructions per 32 columns).  Spilled registers take 4% of those (width 9,
+// class 1: 324 bytes of stores and 372 of loads in the
+// build, 376 and 460 in the adjoint; width 12 about twice, width 5 none to 68).
 // Loading two columns ahead costs the registers of two warps per SM (2.05 ms);
 // 12 and 16 warps per SM are equal.
 #include <algorithm>
